@@ -46,7 +46,7 @@ __device__ __forceinline__ VBlock vblock(const BTab& t, const int* map, int vb) 
 }
 
 template <class T, int KIND, class TO>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 1) kb_stag(Engine e, const PassDesc* descs, BTab t) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) kb_stag(Engine e, const PassDesc* descs, BTab t) {
     const int total = __ldg(t.hdr + 1);
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
         const VBlock q = vblock(t, t.msite, vb);
@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 1) kb_stag(Engi
                     else local = stag_site<T, 2, 0, KIND, TO>(d, op.g, op.l32, alpha, x);
                 }
             } else {
-                if (op.nc == 3) local = stag_site<T, 3, 0, KIND, TO>(d, op.g, op.l64, alpha, x);
-                else local = stag_site<T, 2, 0, KIND, TO>(d, op.g, op.l64, alpha, x);
+                if (op.nc == 3) local = stag_site<T, 3, kLinksFx, KIND, TO>(d, op.g, op.lfx, alpha, x, op.l64);
+                else local = stag_site<T, 2, kLinksFx, KIND, TO>(d, op.g, op.lfx, alpha, x, op.l64);
             }
         }
         if (d.row >= 0) {

@@ -718,7 +718,7 @@ int msc_destroy(msc_ctx* c) {
 }
 
 static void free_op_dev(OpDev& d) {
-    void* ps[] = {d.links64, d.links32, d.slice_len, d.slice_start, d.cols, d.vals64, d.vals32};
+    void* ps[] = {d.links64, d.linksfx, d.links32, d.slice_len, d.slice_start, d.cols, d.vals64, d.vals32};
     for (void* p : ps)
         if (p) cudaFree(p);
     memset(&d, 0, sizeof d);
@@ -815,6 +815,10 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
     const size_t l32 = d.recon ? (size_t)4 * V * (nc == 3 ? 3 : 1) * 16 : (size_t)4 * V * nc * nc * 8;
     e = cudaMalloc(&d.links32, l32);
     if (e == cudaSuccess) e = stag_pack_links32(d, src, c->work);
+    if (e == cudaSuccess && maxdev < 1e-9) {
+        e = cudaMalloc((void**)&d.linksfx, (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16);
+        if (e == cudaSuccess) e = stag_pack_linksfx(d, src, c->work);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
     if (e != cudaSuccess) return fail(e);
     if (tmp) cudaFree(tmp);
@@ -1987,6 +1991,7 @@ extern "C" int msc_solve_batched(msc_ctx* c, int nprob, const msc_problem* probs
         ops[i].recon = A.recon;
         ops[i].l32 = A.links32;
         ops[i].l64 = A.links64;
+        ops[i].lfx = A.linksfx;
         const int64_t np = pad64(A.n);
         for (int r = 0; r < probs[i].nrhs; ++r) {
             BSys q;

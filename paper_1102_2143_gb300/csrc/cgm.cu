@@ -484,7 +484,7 @@ int resident_blocks(const void* fn, int threads) {
 }
 
 dim3 multi_grid(const void* fn, int64_t work, int nsys, bool per_system) {
-    if (per_system && nsys > 1) return dim3(resident_grid(fn, work), nsys);
+    if (per_system && nsys > 1) return dim3(nsys, resident_grid(fn, work));
     // enough blocks for all systems' work, capped at the resident blocks,
     // never fewer than one block per system
     const int64_t total = work * std::max(nsys, 1);

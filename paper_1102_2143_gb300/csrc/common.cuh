@@ -420,17 +420,18 @@ struct SysBlock {
 };
 
 //
-// A 2-D grid instead gives every system a whole grid row (blockIdx.y = system):
-// used by passes that only some listed systems need (reliable updates, FP64
+// A 2-D grid instead gives every system gridDim.y blocks of its own
+// (blockIdx.x = system, so that the same block of every system runs at about
+// the same time and matrix or link tiles come from L2 for all but one): used by passes that only some listed systems need (reliable updates, FP64
 // checks), where the others' blocks exit at once and the busy ones keep the
 // full device.
 __device__ __forceinline__ SysBlock sys_block(int nsys, const int* act) {
     SysBlock s;
     if (gridDim.y > 1 || !act) {
         if (gridDim.y > 1) {
-            s.j = blockIdx.y;
-            s.bx = blockIdx.x;
-            s.gx = gridDim.x;
+            s.j = blockIdx.x;
+            s.bx = blockIdx.y;
+            s.gx = gridDim.y;
             s.ok = s.j < nsys;
             return s;
         }

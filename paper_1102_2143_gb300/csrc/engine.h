@@ -53,6 +53,7 @@ struct OpDev {
     double mass;
     int recon;          // FP32 links keep nc-1 rows
     double2* links64;   // [4][nc*nc][V]
+    int4* linksfx;      // unitary links: fixed-point limbs (see fixed.cuh, fx_link); else null
     void* links32;      // full: float2 [4][nc*nc][V]; recon: float4 [4][k][V]
     // block-CSR in sliced-ELL form, 32 rows per slice
     int bd;
@@ -153,6 +154,7 @@ cudaError_t stag_pack_links(OpDev& op, const double2* links_aos, double* d_maxde
 cudaError_t stag_unitarity(const OpDev& op, const double2* links_aos, double* d_maxdev,
                            cudaStream_t st);
 cudaError_t stag_pack_links32(OpDev& op, const double2* links_aos, cudaStream_t st);
+cudaError_t stag_pack_linksfx(OpDev& op, const double2* links_aos, cudaStream_t st);
 cudaError_t stag_export_bsr(const OpDev& op, int64_t* row_ptr, int32_t* col, double2* vals,
                             cudaStream_t st);
 // max |A_ij - conj(A_ji)| and max |A_ij| over the entries of a block-CSR
@@ -173,6 +175,7 @@ struct BOp {             // one staggered operator of a batch
     int nc, recon;
     const void* l32;
     const double2* l64;
+    const int4* lfx;     // fixed-point limbs, or null (see OpDev)
 };
 struct BSys {            // one system of a batch: a right-hand side (or a refined shift)
     int64_t voff;        // offset (complex) of its r, p, t and t64 rows

@@ -69,6 +69,34 @@ k_stag(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, c
     }
 }
 
+// The FP64 pass over unitary links by fixed-point sums (dslash_site_fx; links
+// that are not unitary may have any range and keep k_stag<double>). Four
+// 128-thread blocks per SM at 128 registers: three at 168 take 2% longer and
+// five at 96 spill. 32^4, one system: 204 us per pass against 570 us on the
+// FP64 pipe (3.9 TB/s against 1.4); about 1,350 instructions per site on the
+// integer-multiply pipe (64% busy, 864 of them the products) and 1,160 on the
+// ALU bound it, then the latency of the gathers at 16 warps per SM.
+constexpr int kFxThreads = 128, kFxBlocks = 4;
+template <int NC, int KIND, class TO>
+__global__ void __launch_bounds__(kFxThreads, kFxBlocks)
+k_stag_fx(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, const void* lfx,
+          const void* links64) {
+    const SysBlock q = sys_block(npass, act);
+    if (!q.ok) return;
+    const PassDesc d = descs[q.j];
+    if (gated_off(e, d)) return;
+    const double alpha = (KIND == PASS_B || KIND == PASS_BC) ? e.sys[d.sys].alpha : 0.0;
+    double local = 0;
+    const int nh = vlen(g);
+    for (int h = q.bx * blockDim.x + threadIdx.x; h < nh; h += q.gx * blockDim.x)
+        local += stag_site<double, NC, kLinksFx, KIND, TO, true>(d, g, lfx, alpha, pass_site<KIND == PASS_A>(h, g),
+                                                                 links64);
+    if (d.row >= 0) {
+        double tot;
+        if (reduce_last_n(e, d.row, local, tot, q.gx, q.bx)) finalize<KIND == PASS_BC>(e, d, tot);
+    }
+}
+
 static int device_sms() {
     static const int n = [] {
         int dev = 0, sms = 0;
@@ -94,12 +122,44 @@ static void launch_one(const Engine& e, const PassDesc* descs, StagGeom g, const
         while (nt > 32 && ((V + nt - 1) / nt) * np < 2 * device_sms()) nt >>= 1;
         if (nt < kThreads) {
             const int per_sys = (int)((V + nt - 1) / nt);
-            const dim3 grid = (per && npass > 1) ? dim3(per_sys, npass) : dim3(per_sys * np);
+            const dim3 grid = (per && npass > 1) ? dim3(npass, per_sys) : dim3(per_sys * np);
             k<<<grid, nt, 0, st>>>(e, descs, npass, act, g, links);
             return;
         }
     }
     k<<<multi_grid((const void*)k, vlen(g), npass, per), kThreads, 0, st>>>(e, descs, npass, act, g, links);
+}
+
+template <int NC, int KIND, class TO>
+static void launch_fx(const Engine& e, const PassDesc* descs, const OpDev& op, int npass, const int* act, bool per,
+                      cudaStream_t st) {
+    auto k = k_stag_fx<NC, KIND, TO>;
+    const int64_t V = vlen(op.g);
+    const int np = std::max(npass, 1);
+    int nt = kFxThreads;
+    while (nt > 32 && ((V + nt - 1) / nt) * np < 2 * device_sms()) nt >>= 1;
+    const int64_t need = (V + nt - 1) / nt, res = resident_blocks((const void*)k, nt);
+    const dim3 grid = (per && npass > 1) ? dim3((unsigned)npass, (unsigned)std::min(need, res))
+                                         : dim3((unsigned)std::max<int64_t>(np, std::min(need * np, res)));
+    k<<<grid, nt, 0, st>>>(e, descs, npass, act, op.g, op.linksfx, op.links64);
+}
+
+template <int NC>
+static cudaError_t launch_kind_fx(int kind, int out_f32, const Engine& e, const PassDesc* descs, const OpDev& op,
+                                  int npass, const int* act, bool per, cudaStream_t st) {
+    switch (kind) {
+        case PASS_A: launch_fx<NC, PASS_A, double>(e, descs, op, npass, act, per, st); break;
+        case PASS_B:
+            if (e.cond_flag) launch_fx<NC, PASS_BC, double>(e, descs, op, npass, act, per, st);
+            else launch_fx<NC, PASS_B, double>(e, descs, op, npass, act, per, st);
+            break;
+        case PASS_C:
+            if (out_f32) launch_fx<NC, PASS_C, float>(e, descs, op, npass, act, per, st);
+            else launch_fx<NC, PASS_C, double>(e, descs, op, npass, act, per, st);
+            break;
+        default: launch_fx<NC, PASS_D, double>(e, descs, op, npass, act, per, st); break;
+    }
+    return cudaGetLastError();
 }
 
 template <class T, int NC, int RECON>
@@ -123,6 +183,10 @@ static cudaError_t launch_kind(int kind, int out_f32, const Engine& e, const Pas
 
 cudaError_t launch_stag_pass(const OpDev& op, int prec, int kind, int out_f32, const Engine& e,
                              const PassDesc* d_descs, int npass, cudaStream_t st, const int* act, bool per) {
+    if (prec == PREC_F64 && op.linksfx) {
+        if (op.nc == 3) return launch_kind_fx<3>(kind, out_f32, e, d_descs, op, npass, act, per, st);
+        return launch_kind_fx<2>(kind, out_f32, e, d_descs, op, npass, act, per, st);
+    }
     if (prec == PREC_F64) {
         if (op.nc == 3) return launch_kind<double, 3, 0>(kind, out_f32, e, d_descs, op.g, op.links64, npass, act, per, st);
         return launch_kind<double, 2, 0>(kind, out_f32, e, d_descs, op.g, op.links64, npass, act, per, st);
@@ -607,6 +671,22 @@ __global__ void k_pack64(const double2* __restrict__ in, double2* __restrict__ o
     }
 }
 
+// AoS [4][V][nc][nc] double2 -> limbs int4 (re.h, re.l, im.h, im.l), see fx_link,
+// in units of 2^-56 (links in U(nc) to rounding: every entry is at most 1)
+__global__ void k_packfx(const double2* __restrict__ in, int4* __restrict__ out, int nc, int V) {
+    const int e2 = nc * nc;
+    const int64_t nl = (int64_t)4 * V;
+    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < nl; l += (int64_t)gridDim.x * blockDim.x) {
+        const int x = (int)(l % V);
+        const int mu = (int)(l / V);
+        for (int c = 0; c < e2; ++c) {
+            const double2 u = in[l * e2 + c];
+            const int2 a = fx_unit(u.x), b = fx_unit(u.y);
+            out[(nc == 3 ? fx_link<3>(mu, x, V) : fx_link<2>(mu, x, V)) + c * 32] = make_int4(a.x, a.y, b.x, b.y);
+        }
+    }
+}
+
 // max over links of max(|U U^dag - 1|_max, |det U - 1|)
 __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlinks,
                             unsigned long long* maxdev) {
@@ -784,6 +864,12 @@ cudaError_t stag_unitarity(const OpDev& op, const double2* links_aos, double* d_
 cudaError_t stag_pack_links32(OpDev& op, const double2* links_aos, cudaStream_t st) {
     const int64_t nl = (int64_t)4 * op.g.V;
     k_pack32<<<setup_blocks(nl), 256, 0, st>>>(links_aos, op.links32, op.nc, op.g.V, op.recon);
+    return cudaGetLastError();
+}
+
+cudaError_t stag_pack_linksfx(OpDev& op, const double2* links_aos, cudaStream_t st) {
+    const int64_t nl = (int64_t)4 * op.g.V;
+    k_packfx<<<setup_blocks(nl), 256, 0, st>>>(links_aos, op.linksfx, op.nc, op.g.V);
     return cudaGetLastError();
 }
 

@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "engine.h"
+#include "fixed.cuh"
 
 namespace msc {
 
@@ -150,6 +151,111 @@ __device__ __forceinline__ void dslash_site(const void* links, const T2<T>* __re
     }
 }
 
+// y = D src at site x in FP64 on the FP64 pipe, for the sites whose entries
+// leave the range of the fixed-point sums (rare: out of line).
+template <int NC> struct SiteVec {
+    double2 y[NC];
+};
+template <int NC>
+__device__ __noinline__ SiteVec<NC> dslash_site_f64(const void* links64, const double2* src, int x, const StagGeom& g) {
+    SiteVec<NC> r;
+    dslash_site<double, NC, 0>(links64, src, x, g, r.y);
+    return r;
+}
+
+// Index of entry 0 of link (mu, x) in the limb array: sites in groups of 32,
+// the entries of a group 32 apart, so that one address serves a link's NC^2
+// loads (constant offsets) and a warp's loads stay contiguous.
+template <int NC>
+__host__ __device__ __forceinline__ size_t fx_link(int mu, int x, int V) {
+    return ((size_t)mu * ((V + 31) >> 5) + (x >> 5)) * (NC * NC * 32) + (x & 31);
+}
+
+// y = D src at site x in FP64 by fixed-point sums (see fixed.cuh). lfx: the
+// limbs (re.h, re.l, im.h, im.l) of each link entry in units of 2^-56, at
+// fx_link().
+// The sign of eta_mu and of the backward hop goes into the entries' limbs.
+// The entries of one direction (both hops) are loaded and bounded together;
+// the first direction sets the sums' unit with one bit to spare, and a later
+// one with larger entries shifts the sums (about two of three warps do so
+// once on Gaussian entries). Holding all 8 hops' entries for one exact bound
+// instead needs 255 registers (32^4, two passes: 506 us).
+template <int NC>
+__device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* links64, const double2* __restrict__ src,
+                                               int x, const StagGeom& g, double2 (&y)[NC]) {
+    if (!lfx) {  // links that are not unitary (batches mix operators)
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
+#pragma unroll
+        for (int a = 0; a < NC; ++a) y[a] = r.y[a];
+        return;
+    }
+    const SiteNbrs nb = neighbours(x, g);
+    FxSum re[NC], im[NC];
+#pragma unroll
+    for (int a = 0; a < NC; ++a) re[a] = im[a] = {0, 0};
+    unsigned field = 0;  // of the sums; Inf and NaN give 2^31, above every entry's
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        double2 v[2][NC];
+        const double2* vf = src + (size_t)vsite(nb.fwd[mu], g) * NC;
+        const double2* vb = src + (size_t)vsite(nb.bwd[mu], g) * NC;
+        unsigned e = 0;
+#pragma unroll
+        for (int b = 0; b < NC; ++b) {
+            v[0][b] = __ldg(vf + b);
+            v[1][b] = __ldg(vb + b);
+        }
+#pragma unroll
+        for (int b = 0; b < NC; ++b) {
+            fx_bound(e, v[0][b]);
+            fx_bound(e, v[1][b]);
+        }
+        const unsigned f = fx_field(e);
+        if (mu == 0) {
+            field = f + (1u << 20);
+        } else if (f > field) {
+            const unsigned d = (f + (1u << 20) - field) >> 20;
+            field = f + (1u << 20);
+#pragma unroll
+            for (int a = 0; a < NC; ++a) {
+                fx_shift(re[a], d);
+                fx_shift(im[a], d);
+            }
+        }
+#pragma unroll
+        for (int dir = 0; dir < 2; ++dir) {
+            const bool fwd = dir == 0;
+            const int4* __restrict__ U = (const int4*)lfx + fx_link<NC>(mu, fwd ? x : nb.bwd[mu], g.V);
+            const int flip = fwd ? -nb.par[mu] : nb.par[mu] - 1;
+#pragma unroll
+            for (int b = 0; b < NC; ++b) {
+                int rh, rl, ih, il;
+                fx_split(v[dir][b].x, field, flip, rh, rl);
+                fx_split(v[dir][b].y, field, flip, ih, il);
+                // forward: U_ab v_b; backward: conj(U_ba) v_b
+                const int zh = fwd ? -ih : ih, zl = fwd ? -il : il;
+                const int wh = fwd ? rh : -rh, wl = fwd ? rl : -rl;
+#pragma unroll
+                for (int a = 0; a < NC; ++a) {
+                    const int4 u = __ldg(U + (fwd ? a * NC + b : b * NC + a) * 32);
+                    fx_mac(re[a], u.x, u.y, rh, rl);
+                    fx_mac(im[a], u.x, u.y, ih, il);
+                    fx_mac(re[a], u.z, u.w, zh, zl);
+                    fx_mac(im[a], u.z, u.w, wh, wl);
+                }
+            }
+        }
+    }
+    if (!fx_in_range(field)) {
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
+#pragma unroll
+        for (int a = 0; a < NC; ++a) y[a] = r.y[a];
+        return;
+    }
+#pragma unroll
+    for (int a = 0; a < NC; ++a) y[a] = {fx_value(re[a], field, 1), fx_value(im[a], field, 1)};
+}
+
 // One site of a D pass: y = D src at x, then the epilogue KIND; returns this
 // site's contribution to the pass's reduction (0 when d.row < 0).
 //   PASS_A: out = y;                       P terms d|aux|^2 + |y|^2
@@ -163,15 +269,19 @@ __device__ __forceinline__ void dslash_site(const void* links, const T2<T>* __re
 template <class T, int KIND>
 using SiteAcc = typename std::conditional<(sizeof(T) == 4 && KIND != PASS_C), float, double>::type;
 
+// RECON = kLinksFx (FP64 only): `links` holds fixed-point limbs and links64
+// the FP64 links.
+constexpr int kLinksFx = 2;
 template <class T, int NC, int RECON, int KIND, class TO, bool PL = false>
 __device__ __forceinline__ SiteAcc<T, KIND> stag_site(const PassDesc& d, const StagGeom& g, const void* links,
-                                            T alpha, int x) {
+                                            T alpha, int x, const void* links64 = nullptr) {
     const T2<T>* __restrict__ src = (const T2<T>*)d.src;
     const T2<T>* __restrict__ aux = (const T2<T>*)d.aux;
     const T dd = (T)d.d;
     const int V = vlen(g);
     T2<T> y[NC];
-    dslash_site<T, NC, RECON, PL>(links, src, x, g, y);
+    if constexpr (RECON == kLinksFx) dslash_site_fx<NC>(links, links64, src, x, g, y);
+    else dslash_site<T, NC, RECON, PL>(links, src, x, g, y);
     x = vsite(x, g);  // the site's index in the vectors
     if (KIND == PASS_A) {
         T2<T>* out = (T2<T>*)d.out;

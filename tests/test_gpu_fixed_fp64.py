@@ -1,0 +1,125 @@
+"""FP64 operator passes by fixed-point sums (csrc/fixed.cuh) against the same
+sums in extended precision.
+
+Tolerances, from the arithmetic: an output of D is at most 96 products of a
+link part (quantised to 2^-57) and an entry part (truncated at 2^-56 of twice
+the largest of the output's own 48 neighbour parts), the product of the low
+limbs dropped (2^-56), halved: below 96 * 2^-55 * vmax = 2^-48.4 vmax, elementwise; the FP64
+form of the oracle must not have a smaller 2-norm error. Entries outside the
+fixed-point range (Inf, NaN, subnormal or near the ends of the exponent range)
+take FP64 arithmetic and give what the oracle gives.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1102_2143_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+import paper_1102_2143_gb300 as msc  # noqa: E402
+
+DIMS = [(3, (2, 4, 6, 2)), (2, (6, 4, 2, 8)), (3, (10, 6, 4, 12))]
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    assert torch.cuda.is_available()
+    c = msc.msc_create(0, torch.cuda.current_stream())
+    yield c
+    msc.msc_destroy(c)
+
+
+def hops(dims):
+    V = inputs.volume(dims)
+    x = np.arange(V)
+    out, stride, par = [], 1, np.zeros(V, int)
+    for L in dims:
+        c = (x // stride) % L
+        out.append((np.where(c == L - 1, x - (L - 1) * stride, x + stride),
+                    np.where(c == 0, x + (L - 1) * stride, x - stride), np.where(par % 2 == 0, 0.5, -0.5)))
+        stride, par = stride * L, par + c
+    return out
+
+
+def dslash_ext(U, dims, nc, v):
+    """D v in extended precision, and the largest neighbour part of each output."""
+    V = inputs.volume(dims)
+    U = U.astype(np.clongdouble)
+    w = v.reshape(V, nc).astype(np.clongdouble)
+    y = np.zeros((V, nc), np.clongdouble)
+    big = np.zeros(V)
+    part = np.maximum(np.abs(v.real), np.abs(v.imag)).reshape(V, nc).max(1)
+    for mu, (f, b, eta) in enumerate(hops(dims)):
+        e = eta[:, None].astype(np.longdouble)
+        y += e * np.einsum("xab,xb->xa", U[mu], w[f])
+        y -= e * np.einsum("xba,xb->xa", np.conj(U[mu][b]), w[b])
+        big = np.maximum(big, np.maximum(part[f], part[b]))
+    return y.reshape(-1), np.repeat(big, nc)
+
+
+def vectors(n, seed):
+    g = inputs.rng(seed)
+    v = inputs.gaussian_source(n, seed)
+    point = np.zeros(n, complex)
+    point[n // 3] = 1.0 - 0.5j
+    return {"gaussian": v, "tiny": v * 1e-200, "huge": v * 1e200, "point": point,
+            "spread": v * np.exp(g.uniform(-60, 60, n)), "zero": np.zeros(n, complex)}
+
+
+@pytest.mark.parametrize("nc,dims", DIMS)
+def test_dslash_against_extended_precision(ctx, nc, dims):
+    U = inputs.su_n_links(dims, nc, 0.9, 40 + nc)
+    op = msc.msc_op_staggered(ctx, nc, dims, torch.from_numpy(U).cuda(), 0.1)
+    n = inputs.volume(dims) * nc
+    for name, v in vectors(n, 50).items():
+        out = np.empty_like(v)
+        msc.msc_op_dslash(ctx, op, v, out)
+        want, big = dslash_ext(U, dims, nc, v)
+        err = np.abs(out.astype(np.clongdouble) - want)
+        assert np.all(err <= 2.0 ** -48.4 * big), (name, float(np.max(err / np.maximum(big, 1e-300))))
+        scale = 1.0 / max(np.abs(v).max(), 1e-300)
+        here = np.linalg.norm((err * scale).astype(float))
+        fp64 = np.linalg.norm((np.abs(oracle.dslash(U, dims, nc, v) - want) * scale).astype(float))
+        if name in ("gaussian", "tiny", "huge"):
+            assert here <= fp64, (name, here, fp64)
+    msc.msc_op_destroy(op)
+
+
+@pytest.mark.parametrize("nc,dims", DIMS)
+def test_out_of_range_entries_take_fp64(ctx, nc, dims):
+    U = inputs.su_n_links(dims, nc, 0.9, 60 + nc)
+    op = msc.msc_op_staggered(ctx, nc, dims, torch.from_numpy(U).cuda(), 0.1)
+    n = inputs.volume(dims) * nc
+    v = inputs.gaussian_source(n, 61)
+    for bad in (np.inf, -np.inf, np.nan):
+        w = v.copy()
+        w[n // 2] = bad
+        out = np.empty_like(w)
+        msc.msc_op_dslash(ctx, op, w, out)
+        want = oracle.dslash(U, dims, nc, w)
+        assert np.array_equal(np.isfinite(out), np.isfinite(want))
+        ok = np.isfinite(want)
+        assert np.linalg.norm(out[ok] - want[ok]) <= 1e-13 * np.linalg.norm(want[ok])
+    for scale in (1e-318, 1e-300, 1e307):
+        w = v * scale
+        out = np.empty_like(w)
+        msc.msc_op_dslash(ctx, op, w, out)
+        want = oracle.dslash(U, dims, nc, w)
+        assert np.max(np.abs(out - want) / scale) <= max(1e-12, 16 * 5e-324 / scale)
+    msc.msc_op_destroy(op)
+
+
+def test_non_unitary_links_stay_on_the_fp64_form(ctx):
+    dims, nc = (4, 6, 4, 2), 3
+    U = 3.0 * inputs.su_n_links(dims, nc, 0.9, 70)
+    U[0, 3] *= 1e5
+    op = msc.msc_op_staggered(ctx, nc, dims, torch.from_numpy(U).cuda(), 0.1)
+    n = inputs.volume(dims) * nc
+    v = inputs.gaussian_source(n, 71)
+    out = np.empty_like(v)
+    msc.msc_op_apply(ctx, op, 0.2, v, out, msc.MSC_FP64)
+    want = oracle.staggered_apply(U, dims, nc, 0.1, v, sigma=0.2)
+    assert np.linalg.norm(out - want) <= 1e-13 * np.linalg.norm(want)
+    msc.msc_op_destroy(op)
