@@ -17,7 +17,8 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
                            const double2* __restrict__ vals, int64_t nbr, int bd,
                            const int32_t* __restrict__ slice_len,
                            const int64_t* __restrict__ slice_start, int32_t* __restrict__ pcol,
-                           double2* __restrict__ v64, float2* __restrict__ v32, int* bad) {
+                           double2* __restrict__ v64, float2* __restrict__ v32, int4* __restrict__ vfx,
+                           uint16_t* __restrict__ efx, int* bad) {
     const int e2 = bd * bd;
     const int64_t nrow_pad = ((nbr + 31) / 32) * 32;
     for (int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; row < nrow_pad;
@@ -33,14 +34,34 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
             int c = 0;
             if (k < rl) {
                 c = col[b0 + k];
-                if (c < 0 || (int64_t)c >= nbr) { atomicExch(bad, 1); c = 0; }
+                if (c < 0 || (int64_t)c >= nbr) { atomicOr(bad, 1); c = 0; }
             }
             pcol[slot * 32 + lane] = c;
+            int ex = 0;
+            if (vfx) {
+                unsigned e = 0;
+                bool zero = true;
+                for (int q = 0; q < e2 && k < rl; ++q) {
+                    const double2 v = vals[(b0 + k) * e2 + q];
+                    fx_bound(e, v);
+                    zero = zero && v.x == 0.0 && v.y == 0.0;
+                }
+                ex = zero ? 0 : (int)(e >> 20);
+                if (!zero && (ex < 200 || ex > 1900)) { atomicOr(bad, 2); ex = 1023; }
+                efx[slot * 32 + lane] = (uint16_t)ex;
+            }
             for (int q = 0; q < e2; ++q) {
                 double2 v = {0.0, 0.0};
                 if (k < rl) v = vals[(b0 + k) * e2 + q];
-                v64[(slot * e2 + q) * 32 + lane] = v;
+                if (v64) v64[(slot * e2 + q) * 32 + lane] = v;
                 v32[(slot * e2 + q) * 32 + lane] = make_float2((float)v.x, (float)v.y);
+                if (vfx) {
+                    // |v| 2^(1022 - ex) < 1, exactly (a power of two)
+                    const double f = __hiloint2double((2045 - ex) << 20, 0);
+                    const int2 a = ex ? fx_unit(v.x * f) : make_int2(0, 0);
+                    const int2 b = ex ? fx_unit(v.y * f) : make_int2(0, 0);
+                    vfx[(slot * e2 + q) * 32 + lane] = make_int4(a.x, a.y, b.x, b.y);
+                }
             }
         }
     }
@@ -107,16 +128,25 @@ cudaError_t bsr_pack(OpDev& op, const int64_t* d_row_ptr, const int32_t* d_col,
     if (b > 65535) b = 65535;
     if (b < 1) b = 1;
     k_bsr_pack<<<(int)b, 256, 0, st>>>(d_row_ptr, d_col, d_vals, op.nbr, op.bd, op.slice_len,
-                                        op.slice_start, op.cols, op.vals64, op.vals32, d_bad);
+                                        op.slice_start, op.cols, op.vals64, op.vals32, op.valsfx, op.blkfx, d_bad);
     return cudaGetLastError();
 }
+
+// FP64 rows by fixed-point sums: three 3 x 3 (four 2 x 2) blocks at a time, three 128-thread
+// blocks per SM (170 registers, no spills). 24^4 (331,776 rows x 33 blocks),
+// one A x: 340 us (4.9 TB/s) against 680 us on the FP64 pipe. Four blocks per
+// SM spill (G = 3: 580 us), or sum one or two blocks at a time (400 / 450 us);
+// two blocks per SM 420 us. The last blocks of a row of 33 are a full group.
+constexpr int kFxRowThreads = 128, kFxRowBlocks = 3;
+template <int BD> constexpr int kFxRowGroup = BD == 3 ? 3 : 4;
 
 // FP32: four 256-thread blocks per SM at up to 64 registers (at five blocks
 // the 48-register cap spills and the 24^4 SpMV takes 160 us instead of
 // 150 us); FP64: three blocks at most 80 registers each: no spills, enough
 // warps for the FP64 pipe.
-template <class T, int BD, int KIND, class TO>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 3)
+// FX (FP64, bd > 1): rows by fixed-point sums (bsr_row_fx), 128-thread blocks.
+template <class T, int BD, int KIND, class TO, bool FX = false>
+__global__ void __launch_bounds__(FX ? kFxRowThreads : kThreads, FX ? kFxRowBlocks : sizeof(T) == 4 ? 4 : 3)
 k_bsr(Engine e, const PassDesc* descs, int npass, const int* act, OpDev A, const T2<T>* __restrict__ vals) {
     const SysBlock q = sys_block(npass, act);
     if (!q.ok) return;
@@ -129,7 +159,8 @@ k_bsr(Engine e, const PassDesc* descs, int npass, const int* act, OpDev A, const
     const int nbr = (int)A.nbr;
     for (int row = q.bx * blockDim.x + threadIdx.x; row < nbr; row += q.gx * blockDim.x) {
         T2<T> y[BD];
-        bsr_row<T, BD>(A, vals, src, row, y);
+        if constexpr (FX) bsr_row_fx<BD, kFxRowGroup<BD>>(A, src, row, y);
+        else bsr_row<T, BD>(A, vals, src, row, y);
         if (KIND == PASS_A) {  // out = (A + d) src, P term = Re src^dag out
             T2<T>* out = (T2<T>*)d.out;
             T loc = T(0);
@@ -346,6 +377,32 @@ static void launch_one(const Engine& e, const PassDesc* descs, const OpDev& A, c
     k<<<multi_grid((const void*)k, A.nbr, npass, per), kThreads, 0, st>>>(e, descs, npass, act, A, vals);
 }
 
+template <int BD, int KIND, class TO>
+static void launch_one_fx(const Engine& e, const PassDesc* descs, const OpDev& A, int npass, const int* act, bool per,
+                          cudaStream_t st) {
+    auto k = k_bsr<double, BD, KIND, TO, true>;
+    const int64_t np = std::max(npass, 1), need = (A.nbr + kFxRowThreads - 1) / kFxRowThreads;
+    const int64_t res = resident_blocks((const void*)k, kFxRowThreads);
+    const dim3 grid = (per && npass > 1) ? dim3((unsigned)np, (unsigned)std::min(need, res))
+                                         : dim3((unsigned)std::max(np, std::min(need * np, res)));
+    k<<<grid, kFxRowThreads, 0, st>>>(e, descs, npass, act, A, nullptr);
+}
+
+template <int BD>
+static cudaError_t launch_bd_fx(int kind, int out_f32, const Engine& e, const PassDesc* descs, const OpDev& A,
+                                int npass, const int* act, bool per, cudaStream_t st) {
+    switch (kind) {
+        case PASS_A: launch_one_fx<BD, PASS_A, double>(e, descs, A, npass, act, per, st); break;
+        case PASS_C:
+            if (out_f32) launch_one_fx<BD, PASS_C, float>(e, descs, A, npass, act, per, st);
+            else launch_one_fx<BD, PASS_C, double>(e, descs, A, npass, act, per, st);
+            break;
+        case PASS_D: launch_one_fx<BD, PASS_D, double>(e, descs, A, npass, act, per, st); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 template <class T, int BD>
 static cudaError_t launch_bd(int kind, int out_f32, const Engine& e, const PassDesc* descs,
                              const OpDev& A, const T2<T>* vals, int npass, const int* act, bool per,
@@ -406,6 +463,10 @@ cudaError_t launch_bsr_pass(const OpDev& op, int prec, int kind, int out_f32, co
     if (kind == PASS_A && npass > 1 && prec == PREC_F32 && !per)
         return launch_bsr_multi(op, e, d_descs, npass, act, kMultiGroup,
                                 (npass + kMultiGroup - 1) / kMultiGroup, st);
+    if (prec == PREC_F64 && op.valsfx) {
+        if (op.bd == 2) return launch_bd_fx<2>(kind, out_f32, e, d_descs, op, npass, act, per, st);
+        return launch_bd_fx<3>(kind, out_f32, e, d_descs, op, npass, act, per, st);
+    }
     if (prec == PREC_F64) {
         switch (op.bd) {
             case 1: return launch_bd<double, 1>(kind, out_f32, e, d_descs, op, op.vals64, npass, act, per, st);

@@ -718,7 +718,7 @@ int msc_destroy(msc_ctx* c) {
 }
 
 static void free_op_dev(OpDev& d) {
-    void* ps[] = {d.links64, d.linksfx, d.links32, d.slice_len, d.slice_start, d.cols, d.vals64, d.vals32};
+    void* ps[] = {d.links64, d.linksfx, d.links32, d.slice_len, d.slice_start, d.cols, d.vals64, d.valsfx, d.blkfx, d.vals32};
     for (void* p : ps)
         if (p) cudaFree(p);
     memset(&d, 0, sizeof d);
@@ -892,7 +892,11 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
     cudaError_t e = cudaMalloc((void**)&d.slice_len, sizeof(int32_t) * nslices);
     if (e == cudaSuccess) e = cudaMalloc((void**)&d.slice_start, sizeof(int64_t) * nslices);
     if (e == cudaSuccess) e = cudaMalloc((void**)&d.cols, sizeof(int32_t) * 32 * std::max<int64_t>(acc, 1));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d.vals64, 16 * e2 * 32 * std::max<int64_t>(acc, 1));
+    // FP64 entries: limbs and block exponents for bd > 1, doubles for bd = 1
+    // (a 1 x 1 block has four FMAs against 36 bytes: nothing to gain)
+    if (e == cudaSuccess && bd > 1) e = cudaMalloc((void**)&d.valsfx, 16 * e2 * 32 * std::max<int64_t>(acc, 1));
+    if (e == cudaSuccess && bd > 1) e = cudaMalloc((void**)&d.blkfx, 2 * 32 * std::max<int64_t>(acc, 1));
+    if (e == cudaSuccess && bd == 1) e = cudaMalloc((void**)&d.vals64, 16 * e2 * 32 * std::max<int64_t>(acc, 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&d.vals32, 8 * e2 * 32 * std::max<int64_t>(acc, 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&trp, sizeof(int64_t) * (nbr + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&dbad, sizeof(int));
@@ -918,7 +922,17 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
     if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, dbad, sizeof(int), cudaMemcpyDeviceToHost, c->work);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
     if (e != cudaSuccess) return fail(cuda_status(e));
-    if (bad) return fail(MSC_ERR_ARG);
+    if (bad & 1) return fail(MSC_ERR_ARG);
+    if (bad) {  // some block does not fit the limbs: the whole matrix in FP64
+        cudaFree(d.valsfx);
+        cudaFree(d.blkfx);
+        d.valsfx = nullptr;
+        d.blkfx = nullptr;
+        e = cudaMalloc((void**)&d.vals64, 16 * e2 * 32 * std::max<int64_t>(acc, 1));
+        if (e == cudaSuccess) e = bsr_pack(d, (const int64_t*)trp, dcol, dval, dbad, c->work);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
+        if (e != cudaSuccess) return fail(cuda_status(e));
+    }
     if (flags & MSC_CHECK_HERMITIAN) {
         // the columns are known to be in range now (the packing checked them)
         double hm[2] = {0.0, 0.0};

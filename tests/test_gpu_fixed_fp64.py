@@ -123,3 +123,77 @@ def test_non_unitary_links_stay_on_the_fp64_form(ctx):
     want = oracle.staggered_apply(U, dims, nc, 0.1, v, sigma=0.2)
     assert np.linalg.norm(out - want) <= 1e-13 * np.linalg.norm(want)
     msc.msc_op_destroy(op)
+
+
+def bsr_ext(rp, ci, va, v, nbr, bd):
+    """A v in extended precision and, per row, the largest block part times
+    entry part summed over its blocks."""
+    w = v.reshape(nbr, bd).astype(np.clongdouble)
+    y = np.zeros((nbr, bd), np.clongdouble)
+    big = np.zeros(nbr)
+    part = np.maximum(np.abs(v.real), np.abs(v.imag)).reshape(nbr, bd).max(1)
+    for i in range(nbr):
+        for k in range(rp[i], rp[i + 1]):
+            y[i] += va[k].astype(np.clongdouble) @ w[ci[k]]
+            big[i] += max(np.abs(va[k].real).max(), np.abs(va[k].imag).max()) * part[ci[k]]
+    return y.reshape(-1), np.repeat(big, bd)
+
+
+@pytest.mark.parametrize("bd,nbr", [(2, 37), (3, 33), (3, 70)])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_bsr_against_extended_precision(ctx, bd, nbr, scaled):
+    """Ragged rows; `scaled`: A -> S A S with S spread over 12 decades and
+    entries over its inverse (products of like size from unlike factors). A
+    group of blocks is summed to 2^-56 of its largest product: an output is
+    within 18 products * 4 * 2^-56 of the sum of the blocks' bounds, plus
+    FP64 roundings of the row sum, below 2^-49 of it."""
+    rp, ci, va, A = inputs.random_hpd_bsr(nbr, bd, 5, 0.5, 80 + nbr)
+    g = inputs.rng(81)
+    s = 10.0 ** g.uniform(-6, 6, nbr) if scaled else np.ones(nbr)
+    for i in range(nbr):
+        for k in range(rp[i], rp[i + 1]):
+            va[k] = va[k] * (s[i] * s[ci[k]])
+    op = msc.msc_op_bsr(ctx, nbr, bd, rp, ci, va)
+    n = nbr * bd
+    v = inputs.gaussian_source(n, 82) / np.repeat(s, bd)
+    for scale in (1.0, 1e-150, 1e150):
+        w = v * scale
+        out = np.empty_like(w)
+        msc.msc_op_apply(ctx, op, 0.0, w, out, msc.MSC_FP64)
+        want, big = bsr_ext(rp, ci, va, w, nbr, bd)
+        err = np.abs(out - want)
+        assert np.all(err <= 2.0 ** -49 * big), float(np.max(err / big))
+        rel = (1.0 / np.repeat(s, bd)) / np.abs(v).max() / scale
+        here = np.linalg.norm((err * rel).astype(float))
+        fp64 = np.linalg.norm((np.abs(oracle.bsr_apply(rp, ci, va, w) - want) * rel).astype(float))
+        assert here <= fp64, (scale, here, fp64)
+    msc.msc_op_destroy(op)
+
+
+@pytest.mark.parametrize("bd", [2, 3])
+def test_bsr_out_of_range_takes_fp64(ctx, bd):
+    nbr = 41
+    rp, ci, va, A = inputs.random_hpd_bsr(nbr, bd, 4, 0.5, 90)
+    n = nbr * bd
+    v = inputs.gaussian_source(n, 91)
+
+    def apply(vals, w):
+        op = msc.msc_op_bsr(ctx, nbr, bd, rp, ci, vals)
+        out = np.empty_like(w)
+        msc.msc_op_apply(ctx, op, 0.0, w, out, msc.MSC_FP64)
+        msc.msc_op_destroy(op)
+        return out
+    w = v.copy()
+    w[n // 2] = np.nan
+    out, want = apply(va, w), oracle.bsr_apply(rp, ci, va, w)
+    # padding blocks read column 0: the others' rows are finite in both
+    assert np.array_equal(np.isfinite(out), np.isfinite(want))
+    for scale_a, scale_v in ((1e250, 1e-310), (1e-250, 1e250), (1e-280, 1.0), (1e290, 1e-5), (1.0, 1e-305)):
+        out, want = apply(va * scale_a, v * scale_v), oracle.bsr_apply(rp, ci, va * scale_a, v * scale_v)
+        tiny = 64 * 5e-324 * max(scale_a, 1.0)
+        assert np.linalg.norm((out - want) / (scale_a * scale_v)) <= \
+            1e-13 * np.linalg.norm(want / (scale_a * scale_v)) + tiny / (scale_a * scale_v), (scale_a, scale_v)
+    b = va.copy()
+    b[3, 0, 0] = np.inf
+    out, want = apply(b, v), oracle.bsr_apply(rp, ci, b, v)
+    assert np.array_equal(np.isfinite(out), np.isfinite(want))
