@@ -242,9 +242,7 @@ __global__ void __launch_bounds__(kThreads) kb_update(Engine e, BVec v, BTab t) 
             const int64_t i = i0 + (int64_t)u * blockDim.x;
             if (i < upv) p[i] = axpy(beta, pv[u], rv[u]);
         }
-        if (arrive_last_n(e, j, w.nb)) {
-            if (threadIdx.x == 0 && s->status == ST_FINISHING) s->status = ST_DONE;
-        }
+        if (st == ST_FINISHING && arrive_last_n(e, j, w.nb)) s->status = ST_DONE;
     }
 }
 

@@ -23,39 +23,28 @@ __device__ __forceinline__ double2 caxpy(double2 a, double2 x, double2 y) {  // 
     return {fma(a.x, x.x, fma(-a.y, x.y, y.x)), fma(a.x, x.y, fma(a.y, x.x, y.y))};
 }
 
-// Three block sums published to rows row0..row0+2; true in every thread of
-// the last block to arrive, with the fixed-order totals.
+// Three block sums published to rows row0..row0+2; true in every lane of warp
+// 0 of the last block to arrive, with the fixed-order totals.
 __device__ bool reduce3_last(const Engine& e, int row0, double a, double b, double c, double (&tot)[3]) {
-    __shared__ double sh[32];
-    __shared__ int is_last;
-    __shared__ double t3[3];
-    const double s0 = block_sum(a, sh), s1 = block_sum(b, sh), s2 = block_sum(c, sh);
-    if (threadIdx.x == 0) {
-        e.partial[(size_t)row0 * kMaxBlocks + blockIdx.x] = s0;
-        e.partial[(size_t)(row0 + 1) * kMaxBlocks + blockIdx.x] = s1;
-        e.partial[(size_t)(row0 + 2) * kMaxBlocks + blockIdx.x] = s2;
-        __threadfence();
-        const unsigned k = atomicAdd(&e.counter[row0], 1u);
-        is_last = (k == gridDim.x - 1);
-    }
+    __shared__ double sv[3][kRedThreads];
     __syncthreads();
-    if (!is_last) return false;
-    __threadfence();
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x)
+    sv[0][threadIdx.x] = a;
+    sv[1][threadIdx.x] = b;
+    sv[2][threadIdx.x] = c;
+    __syncthreads();
+    if (threadIdx.x >= 32) return false;
+    double* part = e.partial + (size_t)row0 * kMaxBlocks;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) acc[q] += __ldcg(&e.partial[(size_t)(row0 + q) * kMaxBlocks + i]);
-    const double u0 = block_sum(acc[0], sh), u1 = block_sum(acc[1], sh), u2 = block_sum(acc[2], sh);
-    if (threadIdx.x == 0) {
-        t3[0] = u0;
-        t3[1] = u1;
-        t3[2] = u2;
-        e.counter[row0] = 0u;
+    for (int q = 0; q < 3; ++q) {
+        const double t = warp_total<double>((int)blockDim.x, [&](int i) { return sv[q][i]; });
+        if (threadIdx.x == 0) part[(size_t)q * kMaxBlocks + blockIdx.x] = t;
     }
-    __syncthreads();
-    tot[0] = t3[0];
-    tot[1] = t3[1];
-    tot[2] = t3[2];
+    int last = 0;
+    if (threadIdx.x == 0) last = arrive(&e.counter[row0]) == gridDim.x - 1;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return false;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) tot[q] = sum_partials(part + (size_t)q * kMaxBlocks, (int)gridDim.x);
+    if (threadIdx.x == 0) e.counter[row0] = 0u;
     return true;
 }
 
@@ -88,7 +77,7 @@ __global__ void __launch_bounds__(kThreads) k_bcg_init(Engine e, BcgSys* sys, Bc
         else if (b2 == 0.0) sys->status = ST_DONE;
     }
     if (b2 == 0.0)
-        for (int k = threadIdx.x; k < S; k += blockDim.x) {
+        for (int k = threadIdx.x; k < S; k += 32) {
             slots[k].active = 0;
             slots[k].conv_iter = 0;
         }
@@ -148,11 +137,9 @@ __global__ void __launch_bounds__(FX ? 128 : kThreads, FX ? 4 : 3) k_bcg_op(OpDe
     const bool ok = isfinite(tt) && cfinite(ts);
     const double2 omega = ok && tt > 0.0 ? double2{ts.x / tt, ts.y / tt} : double2{0.0, 0.0};
     const double2 alpha = sys->alpha, ap = sys->alpha_prev, bp = sys->beta_prev;
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
+    int bad = 0;
     if (ok && tt > 0.0 && !czero(omega)) {
-        for (int k = threadIdx.x; k < S; k += blockDim.x) {
+        for (int k = threadIdx.x; k < S; k += 32) {
             BcgSlot* q = &slots[k];
             if (!q->active) { q->flag = 0; continue; }
             const double sr = q->sigma_rel;
@@ -175,7 +162,7 @@ __global__ void __launch_bounds__(FX ? 128 : kThreads, FX ? 4 : 3) k_bcg_op(OpDe
             if (!cfinite(zn) || !cfinite(Tn) || czero(q->a_s)) bad = 1;
         }
     }
-    __syncthreads();
+    bad = __any_sync(0xffffffffu, bad);
     if (threadIdx.x == 0) {
         if (!ok) sys->status = ST_ERR_NONFINITE;
         else if (!(tt > 0.0) || czero(omega) || bad) sys->status = ST_ERR_BREAKDOWN;
@@ -219,7 +206,7 @@ __global__ void __launch_bounds__(kThreads) k_bcg_r(Engine e, BcgSys* sys, BcgSl
     const double thr = sys->tol2 * sys->bnorm2;
     const int it = sys->it, freeze = sys->freeze;
     int all = 1;
-    for (int k = threadIdx.x; k < S; k += blockDim.x) {
+    for (int k = threadIdx.x; k < S; k += 32) {
         BcgSlot* q = &slots[k];
         if (!q->active) continue;
         const double2 ratio = cdiv(q->zeta_new, q->zeta);
@@ -234,7 +221,7 @@ __global__ void __launch_bounds__(kThreads) k_bcg_r(Engine e, BcgSys* sys, BcgSl
         q->T = q->T_new;
         if (q->conv_iter < 0) all = 0;
     }
-    all = __syncthreads_and(all);
+    all = __all_sync(0xffffffffu, all);
     if (threadIdx.x == 0) {
         sys->rnorm2 = R;
         sys->beta = beta;
@@ -291,16 +278,12 @@ __global__ void __launch_bounds__(kThreads) k_bcg_update(Engine e, BcgSys* sys, 
         // p = r' + beta p - beta omega v
         v.p[i] = caxpy(nbo, v.v[i], caxpy(beta, v.p[i], r1));
     }
-    // the last block retires a finishing system
-    __shared__ int last;
+    // a finishing system is done once every block is
+    if (st != ST_FINISHING) return;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(done_counter, 1u) == gridDim.x - 1;
-        if (last) {
-            *done_counter = 0u;
-            if (sys->status == ST_FINISHING) sys->status = ST_DONE;
-        }
+    if (threadIdx.x == 0 && arrive(done_counter) == gridDim.x - 1) {
+        *done_counter = 0u;
+        sys->status = ST_DONE;
     }
 }
 

@@ -223,9 +223,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_update(Engine e, VecSet v, int 
             if (i < upv) p[i] = axpy(beta, pv[u], rv[u]);
         }
     }
-    if (arrive_last_n(e, j, qb.gx)) {
-        if (threadIdx.x == 0 && s->status == ST_FINISHING) s->status = ST_DONE;
-    }
+    // a finishing system is done once every block is; the others have nothing
+    // to wait for
+    if (st == ST_FINISHING && arrive_last_n(e, j, qb.gx)) s->status = ST_DONE;
 }
 
 // Block-CSR path: r -= alpha Ap and R' = |r|^2 (Algorithm 1, lines 20 and 24).

@@ -72,6 +72,7 @@ struct SlotScalars {
     double sigma_rel;                   // sigma_s - sigma0
     double zeta, zeta_prev, zeta_new;
     double alpha_s, beta_s;
+    double ratio;                       // zeta_new / zeta of this iteration
     int active;                         // still iterating
     int flag;                           // this iteration: 0 skip, 1 x only, 2 x and p_s
     int conv_iter;                      // iteration at which tol was met (-1)
@@ -149,80 +150,184 @@ __device__ __forceinline__ int load_status(const SysScalars* s) {
 }
 
 // ---------------------------------------------------------------------------
-// block reduction + "last block finalizes" (deterministic: fixed-order sums)
+// block reduction + "last block finalizes" (deterministic)
+//
+// An FP64 addition holds an SM's two FP64 lanes for 16 clocks a warp and takes
+// about 100-150 clocks with its shuffle: in a 256-thread block the sum by
+// shuffles in every warp (8 x 5 + 5 additions) and the scalar steps with
+// their divisions in every warp took 5,200-5,500 clocks a step (k_persist,
+// measured). So one warp sums the block's values from shared memory and runs
+// the scalar steps alone, and it adds in fixed point: every value as a 63-bit
+// integer in units of 2^-63 of the power of two above the largest, in two
+// 32-bit limbs whose sums are exact, rounded to FP64 once. (2,000 clocks
+// with FP64 additions by one warp.) The result does not depend on the order,
+// and its error is below n 2^-63 of the largest value, under FP64's own.
 // ---------------------------------------------------------------------------
+constexpr int kRedThreads = 288;  // largest block that reduces
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
 }
 
-// Sum of v over the block, valid in thread 0.
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (w == 0) {
-        t = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
-        t = warp_sum(t);
+// The parts of a float or double as a 63-bit integer of a common exponent.
+template <class T> struct SumBits;
+template <> struct SumBits<float> {
+    static constexpr int kBias = 127 + 23 + 39, kInf = 255;
+    __device__ static __forceinline__ int exponent(float v) { return max((__float_as_int(v) >> 23) & 255, 1); }
+    __device__ static __forceinline__ long long aligned(float v, int top) {
+        const int b = __float_as_int(v), e = (b >> 23) & 255;
+        unsigned long long q = (unsigned long long)((b & 0x7fffff) | (e ? 0x800000 : 0)) << 39;
+        asm("shr.u64 %0, %0, %1;" : "+l"(q) : "r"(top - max(e, 1)));
+        return b < 0 ? -(long long)q : (long long)q;
     }
+};
+template <> struct SumBits<double> {
+    static constexpr int kBias = 1023 + 52 + 10, kInf = 2047;
+    __device__ static __forceinline__ int exponent(double v) { return max((__double2hiint(v) >> 20) & 2047, 1); }
+    __device__ static __forceinline__ long long aligned(double v, int top) {
+        const long long b = __double_as_longlong(v);
+        const int e = (int)(b >> 52) & 2047;
+        unsigned long long q = ((unsigned long long)b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+        q <<= 10;
+        asm("shr.u64 %0, %0, %1;" : "+l"(q) : "r"(top - max(e, 1)));
+        return b < 0 ? -(long long)q : (long long)q;
+    }
+};
+
+// Sum over a warp of 64-bit integers below 2^47 in magnitude, in every lane.
+__device__ __forceinline__ long long warp_add(long long x) {
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0xffffffu);
+    const int hi = __reduce_add_sync(0xffffffffu, (int)(x >> 24));
+    return ((long long)hi << 24) + lo;
+}
+
+// The sum over the warp's lanes of each lane's get(0) .. get(n - 1), in FP64
+// in every lane; top: the largest exponent of this lane's values. K > 0: n = K,
+// unrolled. At most kMaxBlocks values in all. Inf and NaN come out as in FP64
+// additions.
+template <class T, int K, class F>
+__device__ __forceinline__ double warp_total_at(int top, int n, F get) {
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (top == SumBits<T>::kInf) {
+        double acc = 0.0;
+        if constexpr (K > 0) {
+#pragma unroll
+            for (int i = 0; i < K; ++i) acc += (double)get(i);
+        } else {
+            for (int i = 0; i < n; ++i) acc += (double)get(i);
+        }
+        return __shfl_sync(0xffffffffu, warp_sum(acc), 0);
+    }
+    long long hi = 0, lo = 0;
+    auto add = [&](int i) {
+        const long long q = SumBits<T>::aligned(get(i), top);
+        hi += q >> 32;
+        lo += q & 0xffffffffll;
+    };
+    if constexpr (K > 0) {
+#pragma unroll
+        for (int i = 0; i < K; ++i) add(i);
+    } else {
+        for (int i = 0; i < n; ++i) add(i);
+    }
+    hi = warp_add(hi);
+    lo = warp_add(lo);
+    const double r = fma((double)hi, 0x1p32, (double)lo);
+    const int k = top - SumBits<T>::kBias;  // the unit's exponent
+    if (sizeof(T) == 8 && (k < -900 || k > 900)) return scalbn(r, k);
+    return r * __hiloint2double((k + 1023) << 20, 0);
+}
+
+// The sum of get(0) .. get(n - 1), lane by lane.
+template <class T, class F>
+__device__ __forceinline__ double warp_total(int n, F get) {
+    const int lane = threadIdx.x & 31, mine = (n - lane + 31) / 32;
+    int top = 1;
+    for (int i = lane; i < n; i += 32) top = max(top, SumBits<T>::exponent(get(i)));
+    return warp_total_at<T, 0>(top, mine, [&](int i) { return get(lane + 32 * i); });
+}
+
+static __device__ __noinline__ double warp_total_f64(const double* sv, int n) {
+    return warp_total<double>(n, [&](int i) { return sv[i]; });
+}
+
+// Sum of v over the block in FP64, valid in every lane of warp 0. sv:
+// kRedThreads entries of shared memory, free again after the next
+// __syncthreads.
+template <class T>
+__device__ __forceinline__ double block_sum(T v, T* sv) {
     __syncthreads();
+    sv[threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.x >= 32) return 0.0;
+    if constexpr (sizeof(T) == 8) return warp_total_f64(sv, (int)blockDim.x);
+    else return warp_total<T>((int)blockDim.x, [&](int i) { return sv[i]; });
+}
+
+// Sum of n partials, valid in every lane of the calling warp: up to 32 K of
+// them in registers, so that they are read once, all in flight.
+template <int K>
+__device__ __forceinline__ double sum_partials_k(const double* p, int n) {
+    double v[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int i = (threadIdx.x & 31) + 32 * k;
+        v[k] = i < n ? __ldcg(p + i) : 0.0;
+    }
+    int top = 1;
+#pragma unroll
+    for (int k = 0; k < K; ++k) top = max(top, SumBits<double>::exponent(v[k]));
+    return warp_total_at<double, K>(top, K, [&](int k) { return v[k]; });
+}
+// (Out of line, as the FP64 sum below: inlined, their registers make the FP64
+// kernels spill.)
+static __device__ __noinline__ double sum_partials(const double* p, int n) {
+    if (n <= 128) return sum_partials_k<4>(p, n);
+    if (n <= 640) return sum_partials_k<20>(p, n);
+    return warp_total<double>(n, [&](int i) { return __ldcg(p + i); });
+}
+
+// Counts an arrival (one thread): earlier writes of this thread, and of those
+// it has synchronised with, are visible to whoever sees the count.
+__device__ __forceinline__ unsigned arrive(unsigned* counter) {
+    unsigned t;
+    asm volatile("atom.acq_rel.gpu.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
     return t;
 }
 
-// Publishes this block's sum of v to row `row`; returns true in every thread
-// of the last of the `nblocks` blocks that reduce into that row to arrive
-// (`bidx` = this block's index among them), with the fixed-order total.
-__device__ __forceinline__ bool reduce_last_n(const Engine& e, int row, double v, double& total,
-                                              int nblocks, int bidx) {
-    __shared__ double sh[32];
-    __shared__ int is_last;
-    __shared__ double tot;
-    double bs = block_sum(v, sh);
+// Publishes this block's sum of v to row `row`; returns true in every lane of
+// warp 0 of the last of the `nblocks` blocks that reduce into that row to
+// arrive (`bidx` = this block's index among them), with the fixed-order total.
+template <class T>
+__device__ __forceinline__ bool reduce_last_n(const Engine& e, int row, T v, double& total, int nblocks, int bidx) {
+    __shared__ T sv[kRedThreads];
+    const double s = block_sum(v, sv);
+    if (threadIdx.x >= 32) return false;
+    double* part = e.partial + (size_t)row * kMaxBlocks;
+    int last = 0;
     if (threadIdx.x == 0) {
-        e.partial[(size_t)row * kMaxBlocks + bidx] = bs;
-        __threadfence();
-        unsigned t = atomicAdd(&e.counter[row], 1u);
-        is_last = (t == (unsigned)nblocks - 1);
+        part[bidx] = s;
+        last = arrive(&e.counter[row]) == (unsigned)nblocks - 1;
     }
-    __syncthreads();
-    if (!is_last) return false;
-    __threadfence();
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < nblocks; i += blockDim.x)
-        acc += __ldcg(&e.partial[(size_t)row * kMaxBlocks + i]);
-    double s = block_sum(acc, sh);
-    if (threadIdx.x == 0) {
-        tot = s;
-        e.counter[row] = 0u;
-    }
-    __syncthreads();
-    total = tot;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return false;
+    total = sum_partials(part, nblocks);
+    if (threadIdx.x == 0) e.counter[row] = 0u;
     return true;
 }
 
-__device__ __forceinline__ bool reduce_last(const Engine& e, int row, double v, double& total) {
+template <class T>
+__device__ __forceinline__ bool reduce_last(const Engine& e, int row, T v, double& total) {
     return reduce_last_n(e, row, v, total, (int)gridDim.x, (int)blockIdx.x);
 }
 
-// Last block only: signals that every block of a non-reducing kernel is done.
+// True in thread 0 of the last block of a non-reducing kernel to be done.
 __device__ __forceinline__ bool arrive_last_n(const Engine& e, int row, int nblocks) {
-    __shared__ int is_last;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        unsigned t = atomicAdd(&e.counter[row], 1u);
-        is_last = (t == (unsigned)nblocks - 1);
-        if (is_last) e.counter[row] = 0u;
-    }
-    __syncthreads();
-    return is_last != 0;
-}
-
-__device__ __forceinline__ bool arrive_last(const Engine& e, int row) {
-    return arrive_last_n(e, row, (int)gridDim.x);
+    if (threadIdx.x != 0 || arrive(&e.counter[row]) != (unsigned)nblocks - 1) return false;
+    e.counter[row] = 0u;
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -252,29 +357,33 @@ __device__ __forceinline__ float4 to_unit(double2 a, double2 b) {
 }
 
 // ---------------------------------------------------------------------------
-// scalar recurrences, run by the last block (all its threads)
+// scalar recurrences, run by one warp (all its lanes)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void fin_P(const Engine& e, int j, double P) {
+    const int lane = threadIdx.x & 31;
     SysScalars* s = &e.sys[j];
     const double R = s->R, ap = s->alpha_prev, bp = s->beta_prev;
     const int S = s->S, slot0 = s->slot0;
     const bool ok = (P > 0.0) && isfinite(P) && isfinite(R);
     const double alpha = R / P;
-    __syncthreads();
+    __syncwarp();
     if (!ok) {
-        if (threadIdx.x == 0) s->status = isfinite(P) && isfinite(R) ? ST_ERR_NOT_HPD : ST_ERR_NONFINITE;
+        if (lane == 0) s->status = isfinite(P) && isfinite(R) ? ST_ERR_NOT_HPD : ST_ERR_NONFINITE;
         return;
     }
-    for (int k = threadIdx.x; k < S; k += blockDim.x) {
+    for (int k = lane; k < S; k += 32) {
         SlotScalars* q = &e.slot[slot0 + k];
         if (!q->active) { q->flag = 0; continue; }
         const double z = q->zeta, zp = q->zeta_prev;
         const double den = alpha * bp * (zp - z) + zp * ap * (1.0 + q->sigma_rel * alpha);
-        const double zn = z * zp * ap / den;
-        q->zeta_new = zn;
-        q->alpha_s = alpha * zn / z;
+        // zeta'/zeta; exactly 1 for the base shift, whose division would be the
+        // longest chain of a one-shift system
+        const double w = q->sigma_rel == 0.0 && z == zp ? 1.0 : zp * ap / den;
+        q->ratio = w;
+        q->zeta_new = z * w;
+        q->alpha_s = alpha * w;
     }
-    if (threadIdx.x == 0) { s->P = P; s->alpha = alpha; }
+    if (lane == 0) { s->P = P; s->alpha = alpha; }
 }
 
 // COND: this kernel runs inside a chunk graph with conditional update nodes
@@ -282,6 +391,7 @@ __device__ __forceinline__ void fin_P(const Engine& e, int j, double P) {
 // launched elsewhere contain no graph call and stay profilable).
 template <bool COND>
 __device__ __forceinline__ void fin_R(const Engine& e, int j, double Rn) {
+    const int lane = threadIdx.x & 31;
     SysScalars* s = &e.sys[j];
     const double R = s->R, alpha = s->alpha;
     const double thr = s->tol2 * s->bnorm2;
@@ -289,11 +399,11 @@ __device__ __forceinline__ void fin_R(const Engine& e, int j, double Rn) {
     const double beta = Rn / R;
     const bool finite = isfinite(Rn);
     int all = 1;
-    for (int k = threadIdx.x; k < S; k += blockDim.x) {
+    for (int k = lane; k < S; k += 32) {
         SlotScalars* q = &e.slot[slot0 + k];
         if (!q->active) continue;
         const double z = q->zeta, zn = q->zeta_new;
-        const double ratio = zn / z;
+        const double ratio = q->ratio;
         q->beta_s = beta * ratio * ratio;
         const double tk = q->tol2 > 0.0 ? q->tol2 * s->bnorm2 : thr;
         const bool conv = (zn * zn * Rn <= tk) || !(fabs(zn) > 1e-290);
@@ -304,8 +414,8 @@ __device__ __forceinline__ void fin_R(const Engine& e, int j, double Rn) {
         q->zeta = zn;
         if (q->conv_iter < 0) all = 0;
     }
-    all = __syncthreads_and(all);
-    if (threadIdx.x == 0) {
+    all = __all_sync(0xffffffffu, all);
+    if (lane == 0) {
         s->alpha_prev = alpha;
         s->beta_prev = beta;
         s->beta = beta;
@@ -335,24 +445,25 @@ __device__ __forceinline__ void fin_R(const Engine& e, int j, double Rn) {
 // R := reduction. At the start of a solve from a residual, a system that
 // already meets the tolerance is done with nothing to iterate.
 __device__ __forceinline__ void fin_setR(const Engine& e, int j, double Rv, bool init) {
+    const int lane = threadIdx.x & 31;
     SysScalars* s = &e.sys[j];
     const double thr = s->tol2_acc * s->bnorm2;
     const int S = s->S, slot0 = s->slot0;
-    __syncthreads();
+    __syncwarp();
     if (!isfinite(Rv)) {
-        if (threadIdx.x == 0) s->status = ST_ERR_NONFINITE;
+        if (lane == 0) s->status = ST_ERR_NONFINITE;
         return;
     }
     if (init && Rv <= thr) {
-        for (int k = threadIdx.x; k < S; k += blockDim.x) {
+        for (int k = lane; k < S; k += 32) {
             e.slot[slot0 + k].active = 0;
             e.slot[slot0 + k].flag = 0;
             e.slot[slot0 + k].conv_iter = 0;
         }
-        if (threadIdx.x == 0) { s->R = Rv; s->status = ST_DONE; }
+        if (lane == 0) { s->R = Rv; s->status = ST_DONE; }
         return;
     }
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
         s->R = Rv;
         s->Rmax = Rv;
         s->since_ru = 0;
@@ -372,10 +483,11 @@ __device__ __forceinline__ bool fold_skips(const SlotScalars* q, int last_fold) 
 }
 
 __device__ __forceinline__ void fin_init(const Engine& e, int j, double b2) {
+    const int lane = threadIdx.x & 31;
     SysScalars* s = &e.sys[j];
     const int S = s->S, slot0 = s->slot0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    __syncwarp();
+    if (lane == 0) {
         s->R = b2;
         s->Rmax = b2;
         s->since_ru = 0;
@@ -385,7 +497,7 @@ __device__ __forceinline__ void fin_init(const Engine& e, int j, double b2) {
         else if (b2 == 0.0) s->status = ST_DONE;
     }
     if (b2 == 0.0) {
-        for (int k = threadIdx.x; k < S; k += blockDim.x) {
+        for (int k = lane; k < S; k += 32) {
             e.slot[slot0 + k].active = 0;
             e.slot[slot0 + k].conv_iter = 0;
         }
@@ -400,7 +512,7 @@ __device__ __forceinline__ void finalize(const Engine& e, const PassDesc& d, dou
         case FIN_SETR: fin_setR(e, d.sys, total, false); break;
         case FIN_SETR_INIT: fin_setR(e, d.sys, total, true); break;
         case FIN_INIT: fin_init(e, d.sys, total); break;
-        case FIN_STORE: if (threadIdx.x == 0) e.out_red[d.row] = total; break;
+        case FIN_STORE: if ((threadIdx.x & 31) == 0) e.out_red[d.row] = total; break;
         default: break;
     }
 }

@@ -65,7 +65,7 @@ k_stag(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, c
         local += stag_site<T, NC, RECON, KIND, TO, true>(d, g, links, alpha, pass_site<KIND == PASS_A>(h, g));
     if (d.row >= 0) {
         double tot;
-        if (reduce_last_n(e, d.row, (double)local, tot, q.gx, q.bx)) finalize<KIND == PASS_BC>(e, d, tot);
+        if (reduce_last_n(e, d.row, local, tot, q.gx, q.bx)) finalize<KIND == PASS_BC>(e, d, tot);
     }
 }
 
@@ -432,8 +432,8 @@ cudaError_t launch_stag_tile(const OpDev& op, int kind, const Engine& e, const P
 // is that of stag_site (PASS_A: out = D src, P terms; PASS_B/BC: r -= alpha
 // (d aux - D src), |r|^2), and the reductions of a group complete together:
 // its blocks publish one partial per system, then count themselves on the
-// counter of the group's first system; the last block finalizes every
-// system of the group in turn.
+// counter of the group's first system; the last block finalizes the systems
+// of the group, one warp each.
 // ---------------------------------------------------------------------------
 template <int NC, int RECON, int KIND, int NR, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB)
@@ -443,7 +443,7 @@ k_stag_group(Engine e, const PassDesc* descs, int npass, const int* act, StagGeo
     __shared__ PassDesc sd[NR];
     __shared__ float sal[NR];
     __shared__ int son[NR];
-    __shared__ double sred[NR][kThreads / 32];
+    __shared__ float sred[NR][kThreads];
     __shared__ int s_last;
     const int count = act ? __ldg(act) : npass;
     if (count <= 0) return;
@@ -553,42 +553,27 @@ k_stag_group(Engine e, const PassDesc* descs, int npass, const int* act, StagGeo
         }
     }
     if (sd[0].row < 0) return;  // apply-only passes reduce nothing
-    // one partial per system of the group, then the group's arrival count
+    // One partial per system of the group, then the group's arrival count;
+    // warp r sums, and in the last block finalizes, system r, so that the
+    // systems' scalar steps run side by side.
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const double v = warp_sum((double)local[r]);
-        if (lane == 0) sred[r][w] = v;
-    }
+    for (int r = 0; r < NR; ++r) sred[r][threadIdx.x] = local[r];
     __syncthreads();
-    if (w < nr && ((mask >> w) & 1u)) {
-        double t = lane < (int)(blockDim.x >> 5) ? sred[w][lane] : 0.0;
-        t = warp_sum(t);
+    const bool mine = w < nr && ((mask >> w) & 1u);
+    if (mine) {
+        const double t = warp_total<float>((int)blockDim.x, [&](int i) { return sred[w][i]; });
         if (lane == 0) e.partial[(size_t)sd[w].row * kMaxBlocks + bx] = t;
     }
     __syncthreads();
     unsigned* ctr = &e.counter[sd[0].row];
     if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned t = atomicAdd(ctr, 1u);
-        s_last = (t == (unsigned)gx - 1);
+        s_last = arrive(ctr) == (unsigned)gx - 1;
+        if (s_last) *ctr = 0u;
     }
     __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    for (int r = 0; r < nr; ++r) {
-        if (!((mask >> r) & 1u)) continue;
-        const PassDesc d = sd[r];
-        double acc = 0.0;
-        for (int i = threadIdx.x; i < gx; i += blockDim.x) acc += __ldcg(&e.partial[(size_t)d.row * kMaxBlocks + i]);
-        const double tot = block_sum(acc, &sred[0][0]);
-        __shared__ double s_tot;
-        if (threadIdx.x == 0) s_tot = tot;
-        __syncthreads();
-        finalize<KIND == PASS_BC>(e, d, s_tot);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *ctr = 0u;
+    if (!s_last || !mine) return;
+    finalize<KIND == PASS_BC>(e, sd[w], sum_partials(e.partial + (size_t)sd[w].row * kMaxBlocks, gx));
 }
 
 template <int NC, int RECON, int NR, int MINB>
