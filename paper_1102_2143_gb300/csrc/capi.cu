@@ -62,6 +62,9 @@ struct Range {
 
 }  // namespace
 
+// small results of the set-up kernels, behind the context's error word
+constexpr size_t kSetupWord = 4, kSetupMax = 8;
+
 struct msc_ctx {
     int device = 0;
     int num_sms = 0;
@@ -78,7 +81,9 @@ struct msc_ctx {
     Buf bcg;          // BiCGStab-M scalars: one BcgSys, then S BcgSlot
     Buf condf;        // one flag per iteration of a chunk graph (conditional update bodies)
     Buf pb, px0, ptmp;// polynomial right-hand sides: b_s, x_s0, two scratch vectors per shift
-    Buf errf;         // device error word (bit 0: a bounded wait in a kernel ran out)
+    Buf gbar;         // barrier word of the cooperative iterations
+    Buf errf;         // device error word (bit 0: a bounded wait in a kernel ran out), then
+                      // scratch words of the operators' set-up (offsets kSetupWord, kSetupMax)
     unsigned* h_err = nullptr;  // pinned copy of it
     uint64_t wait_ns = 2000000000ull;  // limit of a kernel's wait on its own copies
     int use_tile = 0;  // one-system FP32 stencil passes stage their links (when the lattice tiles)
@@ -477,6 +482,61 @@ struct ProfAcc {
     int n = 0;
 };
 
+// A stage of small staggered systems: cooperative launches that each run
+// iterations until the systems stop or one is due a reliable update
+// (persist.cu), every one followed by the gated kernels of that update. No
+// graph: a handful of launches per update, and nothing to instantiate for a
+// new operator. c->h_sys holds the systems' scalars.
+static int run_stage_persist(msc_ctx* c, const msc_op* op, int prec, int nsys, int nslots, bool reliable, int64_t npad,
+                             int max_iter, int* rel_updates) {
+    const OpDev& A = op->dev;
+    bool moved = false;
+    CK(grow(c, c->gbar, 256, moved));
+    PersistArgs a;
+    a.e = engine_of(c);
+    a.v = vecs_of(c, prec, npad, A);
+    a.k1 = dsec(c, D_K1);
+    a.k2 = dsec(c, D_K2);
+    a.g = A.g;
+    a.links = prec == PREC_F64 ? (const void*)A.linksfx : A.links32;
+    a.links64 = A.links64;
+    a.bar = (unsigned*)c->gbar.p;
+    a.wait_ns = c->wait_ns;
+    a.nsys = nsys;
+    a.nslots = nslots;
+    a.iters = reliable ? 50 : 100;
+    const int reps = reliable ? 4 : 1;  // launches between two looks at the status
+    // every launch but the last of a stage ends in an iteration or an update
+    const long most = max_iter > 0 ? 2L * max_iter + 8 : 0;
+    for (long k = 0; k < most; ++k) {
+        bool any = false;
+        for (int j = 0; j < nsys; ++j) any = any || c->h_sys[j].status < ST_DONE;
+        if (!any) break;
+        for (int q = 0; q < reps; ++q) {
+            CK(cudaMemsetAsync(c->gbar.p, 0, sizeof(unsigned), c->work));
+            CK(launch_persist(A, prec, a, c->work));
+            c->launches++;
+            if (!reliable) continue;
+            CK(launch_fold(a.e, a.v, nsys, 1, c->work, nullptr, true));
+            CK(op_pass(c, A, PREC_F64, PASS_A, 0, D_RUA, nsys, &a.e, nullptr, true));
+            CK(op_pass(c, A, PREC_F64, PASS_C, 1, D_RUC, nsys, &a.e, nullptr, true));
+            c->launches++;
+        }
+        CK(cudaMemcpyAsync(c->h_sys, c->sys.p, sizeof(SysScalars) * nsys, cudaMemcpyDeviceToHost, c->work));
+        CK(cudaMemcpyAsync(c->h_err, c->errf.p, sizeof(unsigned), cudaMemcpyDeviceToHost, c->work));
+        CK(cudaStreamSynchronize(c->work));
+        if (*c->h_err) {
+            // a barrier's bounded wait ran out: the launch's results are void
+            CK(cudaMemsetAsync(c->errf.p, 0, sizeof(unsigned), c->work));
+            CK(cudaStreamSynchronize(c->work));
+            return MSC_ERR_TIMEOUT;
+        }
+    }
+    if (rel_updates)
+        for (int j = 0; j < nsys; ++j) *rel_updates += c->h_sys[j].nru;
+    return MSC_OK;
+}
+
 // Launch chunks until every system has stopped. With `compact` (several
 // systems sharing a block-CSR matrix in FP32), the SpMV of each chunk runs
 // only the systems still iterating, in groups sized for their number.
@@ -495,6 +555,14 @@ static int run_stage(msc_ctx* c, const msc_op* op, int prec, int nsys, int chunk
             c->h_act_cap = nsys + 1;
         }
     }
+    CK(cudaMemcpyAsync(c->h_sys, c->sys.p, sizeof(SysScalars) * nsys, cudaMemcpyDeviceToHost, c->work));
+    CK(cudaStreamSynchronize(c->work));
+    int nslot_all = 0;
+    for (int j = 0; j < nsys; ++j) nslot_all = std::max(nslot_all, c->h_sys[j].slot0 + c->h_sys[j].S);
+    const bool tiled = c->use_tile && nsys == 1 && prec == PREC_F32 && op->dev.kind == OP_STAGGERED && op->dev.recon &&
+                       stag_tile_fits(op->dev.g, op->dev.nc);
+    if (!tiled && persist_applies(op->dev, prec, nsys, nslot_all))
+        return run_stage_persist(c, op, prec, nsys, nslot_all, reliable, npad, max_iter, rel_updates);
     GraphEntry* ge = nullptr;
     int st = MSC_OK;
     if (!compact) {
@@ -504,13 +572,9 @@ static int run_stage(msc_ctx* c, const msc_op* op, int prec, int nsys, int chunk
                        multi ? (nsys + kMultiGroup - 1) / kMultiGroup : 0, &ge);
         if (st != MSC_OK) return st;
     }
-    CK(cudaMemcpyAsync(c->h_sys, c->sys.p, sizeof(SysScalars) * nsys, cudaMemcpyDeviceToHost, c->work));
-    CK(cudaStreamSynchronize(c->work));
     // profiled stages: the non-base shifts still iterating when a chunk
     // starts (the shifts its first, sampled, update kernel moves)
     const bool track = profile && pa;
-    int nslot_all = 0;
-    for (int j = 0; j < nsys; ++j) nslot_all = std::max(nslot_all, c->h_sys[j].slot0 + c->h_sys[j].S);
     auto count_active = [&]() {
         int a = 0;
         for (int j = 0; j < nsys; ++j)
@@ -699,7 +763,7 @@ int msc_destroy(msc_ctx* c) {
     Buf* bufs[] = {&c->sys, &c->slot, &c->partial, &c->counter, &c->out_red, &c->descs,
                    &c->b64, &c->x64, &c->t64, &c->r, &c->p, &c->t, &c->ps, &c->xit,
                    &c->coef, &c->force, &c->btab, &c->actb, &c->condf, &c->bcg,
-                   &c->pb, &c->px0, &c->ptmp, &c->errf};
+                   &c->pb, &c->px0, &c->ptmp, &c->gbar, &c->errf};
     for (Buf* b : bufs)
         if (b->p) cudaFree(b->p);
     if (c->h_sys) cudaFreeHost(c->h_sys);
@@ -718,7 +782,8 @@ int msc_destroy(msc_ctx* c) {
 }
 
 static void free_op_dev(OpDev& d) {
-    void* ps[] = {d.links64, d.linksfx, d.links32, d.slice_len, d.slice_start, d.cols, d.vals64, d.valsfx, d.blkfx, d.vals32};
+    // links64 holds the staggered operator's one allocation
+    void* ps[] = {d.links64, d.slice_len, d.slice_start, d.cols, d.vals64, d.valsfx, d.blkfx, d.vals32};
     for (void* p : ps)
         if (p) cudaFree(p);
     memset(&d, 0, sizeof d);
@@ -787,11 +852,10 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
     const size_t nlink_bytes = (size_t)4 * V * nc * nc * 16;
     const double2* src = (const double2*)links;
     void* tmp = nullptr;
-    double* dmax = nullptr;
+    double* dmax = (double*)((char*)c->errf.p + kSetupMax);
     cudaError_t e = cudaSuccess;
     auto fail = [&](cudaError_t err) {
         if (tmp) cudaFree(tmp);
-        if (dmax) cudaFree(dmax);
         free_op_dev(d);
         delete op;
         return cuda_status(err);
@@ -802,10 +866,7 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
         if (e != cudaSuccess) return fail(e);
         src = (const double2*)tmp;
     }
-    e = cudaMalloc((void**)&d.links64, nlink_bytes);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&dmax, sizeof(double));
-    if (e == cudaSuccess) e = cudaMemsetAsync(dmax, 0, sizeof(double), c->work);
-    if (e == cudaSuccess) e = stag_pack_links(d, src, dmax, c->work);
+    e = cudaMemsetAsync(dmax, 0, sizeof(double), c->work);
     if (e == cudaSuccess) e = stag_unitarity(d, src, dmax, c->work);
     double maxdev = 1.0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&maxdev, dmax, sizeof(double), cudaMemcpyDeviceToHost, c->work);
@@ -813,16 +874,22 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
     if (e != cudaSuccess) return fail(e);
     d.recon = (!(flags & MSC_LINKS_FULL) && maxdev < 1e-9) ? 1 : 0;
     const size_t l32 = d.recon ? (size_t)4 * V * (nc == 3 ? 3 : 1) * 16 : (size_t)4 * V * nc * nc * 8;
-    e = cudaMalloc(&d.links32, l32);
+    const size_t lfx = maxdev < 1e-9 ? (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16 : 0;
+    // one allocation for the three forms (each cudaMalloc and cudaFree costs
+    // tens of microseconds of a small operator's set-up): FP64, limbs, FP32
+    const size_t at_fx = (nlink_bytes + 255) / 256 * 256, at_32 = at_fx + (lfx + 255) / 256 * 256;
+    char* block = nullptr;
+    e = cudaMalloc((void**)&block, at_32 + l32);
+    if (e != cudaSuccess) return fail(e);
+    d.links64 = (double2*)block;
+    d.linksfx = lfx ? (int4*)(block + at_fx) : nullptr;
+    d.links32 = block + at_32;
+    e = stag_pack_links(d, src, dmax, c->work);
     if (e == cudaSuccess) e = stag_pack_links32(d, src, c->work);
-    if (e == cudaSuccess && maxdev < 1e-9) {
-        e = cudaMalloc((void**)&d.linksfx, (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16);
-        if (e == cudaSuccess) e = stag_pack_linksfx(d, src, c->work);
-    }
+    if (e == cudaSuccess && lfx) e = stag_pack_linksfx(d, src, c->work);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
     if (e != cudaSuccess) return fail(e);
     if (tmp) cudaFree(tmp);
-    cudaFree(dmax);
     *out = op;
     return MSC_OK;
 }
@@ -876,13 +943,12 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
     d.nslices = nslices;
     d.nslots_blk = acc;
     void *trp = nullptr, *tcol = nullptr, *tval = nullptr;
-    int* dbad = nullptr;
+    int* dbad = (int*)((char*)c->errf.p + kSetupWord);
     unsigned long long* dherm = nullptr;
     auto fail = [&](int code) {
         if (trp) cudaFree(trp);
         if (tcol) cudaFree(tcol);
         if (tval) cudaFree(tval);
-        if (dbad) cudaFree(dbad);
         if (dherm) cudaFree(dherm);
         free_op_dev(d);
         delete op;
@@ -899,7 +965,6 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
     if (e == cudaSuccess && bd == 1) e = cudaMalloc((void**)&d.vals64, 16 * e2 * 32 * std::max<int64_t>(acc, 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&d.vals32, 8 * e2 * 32 * std::max<int64_t>(acc, 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&trp, sizeof(int64_t) * (nbr + 1));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&dbad, sizeof(int));
     if (e != cudaSuccess) return fail(cuda_status(e));
     e = cudaMemcpyAsync(d.slice_len, slen.data(), sizeof(int32_t) * nslices, cudaMemcpyHostToDevice, c->work);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d.slice_start, sstart.data(), sizeof(int64_t) * nslices, cudaMemcpyHostToDevice, c->work);
@@ -949,7 +1014,6 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
     cudaFree(trp);
     if (tcol) cudaFree(tcol);
     if (tval) cudaFree(tval);
-    cudaFree(dbad);
     *out = op;
     return MSC_OK;
 }

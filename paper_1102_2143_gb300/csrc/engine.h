@@ -122,6 +122,26 @@ struct VecSet {
     int pl_nc = 0;
     int pl_V = 0;
 };
+// Iterations of small staggered systems in one cooperative launch
+// (persist.cu): all nsys systems (whose shifts lie in the first nslots slots)
+// run until every one has stopped, one of them is due a reliable update, or
+// `iters` iterations are done. k1, k2: the pass descriptors (device). bar: a
+// barrier word, zeroed before each launch. persist_applies() says whether a
+// stage takes this path.
+struct PersistArgs {
+    Engine e;
+    VecSet v;
+    const PassDesc* k1;
+    const PassDesc* k2;
+    StagGeom g;
+    const void* links;
+    const void* links64;
+    unsigned* bar;
+    uint64_t wait_ns;
+    int nsys, nslots, iters;
+};
+bool persist_applies(const OpDev& op, int prec, int nsys, int nslots);
+cudaError_t launch_persist(const OpDev& op, int prec, const PersistArgs& a, cudaStream_t st);
 cudaError_t launch_init(int prec, const Engine& e, const VecSet& v, const PassDesc* d_descs,
                         int nsys, cudaStream_t st);
 cudaError_t launch_init_from_r(int prec, const Engine& e, const VecSet& v, int nsys, cudaStream_t st);

@@ -180,7 +180,9 @@ __host__ __device__ __forceinline__ size_t fx_link(int mu, int x, int V) {
 // one with larger entries shifts the sums (about two of three warps do so
 // once on Gaussian entries). Holding all 8 hops' entries for one exact bound
 // instead needs 255 registers (32^4, two passes: 506 us).
-template <int NC>
+// FRESH: src may have been written by other blocks of the same kernel, so its
+// loads do not take the read-only path.
+template <int NC, bool FRESH>
 __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* links64, const double2* __restrict__ src,
                                                int x, const StagGeom& g, double2 (&y)[NC]) {
     if (!lfx) {  // links that are not unitary (batches mix operators)
@@ -202,8 +204,8 @@ __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* link
         unsigned e = 0;
 #pragma unroll
         for (int b = 0; b < NC; ++b) {
-            v[0][b] = __ldg(vf + b);
-            v[1][b] = __ldg(vb + b);
+            v[0][b] = FRESH ? vf[b] : __ldg(vf + b);
+            v[1][b] = FRESH ? vb[b] : __ldg(vb + b);
         }
 #pragma unroll
         for (int b = 0; b < NC; ++b) {
@@ -272,7 +274,7 @@ using SiteAcc = typename std::conditional<(sizeof(T) == 4 && KIND != PASS_C), fl
 // RECON = kLinksFx (FP64 only): `links` holds fixed-point limbs and links64
 // the FP64 links.
 constexpr int kLinksFx = 2;
-template <class T, int NC, int RECON, int KIND, class TO, bool PL = false>
+template <class T, int NC, int RECON, int KIND, class TO, bool PL = false, bool FRESH = false>
 __device__ __forceinline__ SiteAcc<T, KIND> stag_site(const PassDesc& d, const StagGeom& g, const void* links,
                                             T alpha, int x, const void* links64 = nullptr) {
     const T2<T>* __restrict__ src = (const T2<T>*)d.src;
@@ -280,7 +282,7 @@ __device__ __forceinline__ SiteAcc<T, KIND> stag_site(const PassDesc& d, const S
     const T dd = (T)d.d;
     const int V = vlen(g);
     T2<T> y[NC];
-    if constexpr (RECON == kLinksFx) dslash_site_fx<NC>(links, links64, src, x, g, y);
+    if constexpr (RECON == kLinksFx) dslash_site_fx<NC, FRESH>(links, links64, src, x, g, y);
     else dslash_site<T, NC, RECON, PL>(links, src, x, g, y);
     x = vsite(x, g);  // the site's index in the vectors
     if (KIND == PASS_A) {
