@@ -82,13 +82,15 @@ __device__ __forceinline__ int2 fx_unit(double u) {
     return q < 0 ? make_int2(-h, -l) : make_int2(h, l);
 }
 
-// The sum of products of unit factors and entries of exponent field `field`,
-// times 2^-half.
-__device__ __forceinline__ double fx_value(const FxSum& s, unsigned field, int half) {
-    const long long t = s.h + ((s.m + (1 << 27)) >> 28);
+// t units of the sum of products of unit factors and entries of exponent field
+// `field`, times 2^-half.
+__device__ __forceinline__ double fx_double(long long t, unsigned field, int half) {
     const double d = (double)t;
     const int hi = __double2hiint(d) + (int)field - ((1078 + half) << 20);
     return t == 0 ? 0.0 : __hiloint2double(hi, __double2loint(d));
+}
+__device__ __forceinline__ double fx_value(const FxSum& s, unsigned field, int half) {
+    return fx_double(s.h + ((s.m + (1 << 27)) >> 28), field, half);
 }
 
 }  // namespace msc

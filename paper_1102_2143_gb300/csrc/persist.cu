@@ -20,8 +20,7 @@
 // Measured, one system, mixed, per iteration: 4^4 with 8 shifts 37 -> 12 us,
 // 16^4 with one shift 29 -> 18 us (of which three barriers 3.8, the scalar
 // steps 3.7, the passes with their sums 7); the 4^4 8-shift solve 15.0 ->
-// 5.4 ms. FP64 (fixed-point passes) 8^4: 28 us, bound by the passes' latency
-// at one or two warps per scheduler.
+// 5.4 ms. FP64 (fixed-point passes): 4^4 16 us, 8^4 17 us.
 //
 // Barrier waits are bounded by the global timer (wait_ns): a wait that runs
 // out sets the context's error word and the block returns.
@@ -129,10 +128,16 @@ __device__ __forceinline__ void copy_words(D* to, const D* from, int count) {
 
 constexpr int kShiftBatch = 4;  // shifts whose loads are in flight together in the update
 
-// BPS blocks per SM: FP64 at one (255 registers) when no more blocks are wanted
-// than SMs (8^4: 27.6 us an iteration against 32.7 at two, which spill), at two
-// otherwise (16^4: 44.9 against 47.0).
-template <class T, int NC, int RECON, int BPS>
+// FX4 (FP64): four lanes share a site (stag_site_fx4), 64 sites to a task
+// instead of 256. Chosen up to kFx4PersistSites sites of all systems, where a
+// pass is the latency of one site's instructions: 8^4 16.9 us an iteration
+// against 27.6, 4 x 8^4 24.0 against 27.8, but 12^4 31.9 against 27.6.
+// BPS blocks per SM: FP64 with a thread per site at one (255 registers) when no
+// more blocks are wanted than SMs (8^4: 27.6 us against 32.7 at two, which
+// spill), at two otherwise (16^4: 44.9 against 47.0).
+constexpr int64_t kFx4PersistSites = 16384;
+
+template <class T, int NC, int RECON, int BPS, bool FX4>
 __global__ void __launch_bounds__(kThreads, BPS) k_persist(PersistArgs a) {
     using V = typename U16<T>::t;
     extern __shared__ unsigned long long dyn[];
@@ -154,7 +159,8 @@ __global__ void __launch_bounds__(kThreads, BPS) k_persist(PersistArgs a) {
     e.slot = sl;
     const StagGeom& g = a.g;
     const int nh = vlen(g);
-    const int chunks = (nh + kThreads - 1) / kThreads;
+    constexpr int kSites = FX4 ? kThreads / 4 : kThreads;
+    const int chunks = (nh + kSites - 1) / kSites;
     const int ntask = nsys * chunks;
     const int64_t upv = a.v.npad / U16<T>::cpu;
     const int vchunks = (int)((upv + kThreads - 1) / kThreads);
@@ -172,11 +178,17 @@ __global__ void __launch_bounds__(kThreads, BPS) k_persist(PersistArgs a) {
         for (int q = blockIdx.x; q < ntask; q += gridDim.x) {
             const int j = q / chunks, ch = q - j * chunks;
             if (ss[j].status != ST_RUNNING) continue;
-            const int h = ch * kThreads + threadIdx.x;
             SiteAcc<T, PASS_A> local = 0;
-            if (h < nh)
-                local = stag_site<T, NC, RECON, PASS_A, T, true, true>(k1[j], g, a.links, T(0),
-                                                                       pass_site<true>(h, g), a.links64);
+            if constexpr (FX4) {
+                const int h = ch * kSites + (threadIdx.x >> 2);
+                local = stag_site_fx4<NC, PASS_A, double, true>(k1[j], g, a.links, a.links64, T(0),
+                                                                 pass_site<true>(h < nh ? h : 0, g), h < nh);
+            } else {
+                const int h = ch * kSites + threadIdx.x;
+                if (h < nh)
+                    local = stag_site<T, NC, RECON, PASS_A, T, true, true>(k1[j], g, a.links, T(0),
+                                                                           pass_site<true>(h, g), a.links64);
+            }
             const double s = block_sum(local, sv);
             if (threadIdx.x == 0) e.partial[(size_t)j * kMaxBlocks + ch] = s;
         }
@@ -188,11 +200,17 @@ __global__ void __launch_bounds__(kThreads, BPS) k_persist(PersistArgs a) {
         for (int q = blockIdx.x; q < ntask; q += gridDim.x) {
             const int j = q / chunks, ch = q - j * chunks;
             if (ss[j].status != ST_RUNNING) continue;
-            const int h = ch * kThreads + threadIdx.x;
             SiteAcc<T, PASS_B> local = 0;
-            if (h < nh)
-                local = stag_site<T, NC, RECON, PASS_B, T, true, true>(k2[j], g, a.links, cy[j].alpha,
-                                                                       pass_site<false>(h, g), a.links64);
+            if constexpr (FX4) {
+                const int h = ch * kSites + (threadIdx.x >> 2);
+                local = stag_site_fx4<NC, PASS_B, double, true>(k2[j], g, a.links, a.links64, cy[j].alpha,
+                                                                 pass_site<false>(h < nh ? h : 0, g), h < nh);
+            } else {
+                const int h = ch * kSites + threadIdx.x;
+                if (h < nh)
+                    local = stag_site<T, NC, RECON, PASS_B, T, true, true>(k2[j], g, a.links, cy[j].alpha,
+                                                                           pass_site<false>(h, g), a.links64);
+            }
             const double s = block_sum(local, sv);
             if (threadIdx.x == 0) e.partial[(size_t)j * kMaxBlocks + kHalfRow + ch] = s;
         }
@@ -278,16 +296,30 @@ bool persist_applies(const OpDev& op, int prec, int nsys, int nslots) {
     return nsys * chunks <= kPersistTasks && chunks <= kHalfRow && persist_smem(nsys, nslots) <= 40 * 1024;
 }
 
-template <class T, int NC, int RECON, int BPS>
-static cudaError_t launch_persist_t(PersistArgs a, int sms, int64_t tasks, cudaStream_t st) {
-    auto k = k_persist<T, NC, RECON, BPS>;
+template <class T, int NC, int RECON, int BPS, bool FX4 = false>
+static cudaError_t launch_persist_t(PersistArgs a, int sms, cudaStream_t st) {
+    auto k = k_persist<T, NC, RECON, BPS, FX4>;
     const size_t sm = persist_smem(a.nsys, a.nslots);
     int per_sm = 0;
     cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k, kThreads, sm);
     if (err != cudaSuccess) return err;
+    const int sites = FX4 ? kThreads / 4 : kThreads;
+    const int64_t tasks = a.nsys * (int64_t)((vlen(a.g) + sites - 1) / sites);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tasks, (int64_t)per_sm * sms));
     void* ptrs[] = {&a};
     return cudaLaunchCooperativeKernel((const void*)k, dim3(grid), dim3(kThreads), ptrs, sm, st);
+}
+
+template <int NC>
+static cudaError_t launch_persist_nc(const OpDev& op, int prec, const PersistArgs& a, int sms, cudaStream_t st) {
+    if (prec == PREC_F64) {
+        const int64_t V = vlen(a.g);
+        if (a.nsys * V <= kFx4PersistSites) return launch_persist_t<double, NC, kLinksFx, 2, true>(a, sms, st);
+        if (a.nsys * ((V + kThreads - 1) / kThreads) <= sms) return launch_persist_t<double, NC, kLinksFx, 1>(a, sms, st);
+        return launch_persist_t<double, NC, kLinksFx, 2>(a, sms, st);
+    }
+    if (op.recon) return launch_persist_t<float, NC, 1, 2>(a, sms, st);
+    return launch_persist_t<float, NC, 0, 2>(a, sms, st);
 }
 
 cudaError_t launch_persist(const OpDev& op, int prec, const PersistArgs& a, cudaStream_t st) {
@@ -295,17 +327,7 @@ cudaError_t launch_persist(const OpDev& op, int prec, const PersistArgs& a, cuda
     cudaError_t err = cudaGetDevice(&dev);
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    const int64_t tasks = a.nsys * (int64_t)((vlen(a.g) + kThreads - 1) / kThreads);
-    const bool n3 = op.nc == 3;
-    if (prec == PREC_F64 && tasks <= sms)
-        return n3 ? launch_persist_t<double, 3, kLinksFx, 1>(a, sms, tasks, st)
-                  : launch_persist_t<double, 2, kLinksFx, 1>(a, sms, tasks, st);
-    if (prec == PREC_F64)
-        return n3 ? launch_persist_t<double, 3, kLinksFx, 2>(a, sms, tasks, st)
-                  : launch_persist_t<double, 2, kLinksFx, 2>(a, sms, tasks, st);
-    if (op.recon)
-        return n3 ? launch_persist_t<float, 3, 1, 2>(a, sms, tasks, st) : launch_persist_t<float, 2, 1, 2>(a, sms, tasks, st);
-    return n3 ? launch_persist_t<float, 3, 0, 2>(a, sms, tasks, st) : launch_persist_t<float, 2, 0, 2>(a, sms, tasks, st);
+    return op.nc == 3 ? launch_persist_nc<3>(op, prec, a, sms, st) : launch_persist_nc<2>(op, prec, a, sms, st);
 }
 
 }  // namespace msc

@@ -97,6 +97,36 @@ k_stag_fx(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g
     }
 }
 
+// The same with four lanes per site (stag_site_fx4).
+// Chosen up to kFx4Sites sites in all, where a pass is the latency of the 2,700
+// instructions of a site on a warp or two per scheduler. One A x (two
+// passes) in a graph, four lanes against one: 4^4 7.7 against 14.7 us, 8^4 8.5
+// against 15.1, 12^4 16.3 against 18.8, but 14^4 20.9 against 20.0 and 32^4 485
+// against 410 (more instructions in all).
+constexpr int kFx4Threads = 128;
+constexpr int64_t kFx4Sites = 24576;
+template <int NC, int KIND, class TO>
+__global__ void __launch_bounds__(kFx4Threads, kFxBlocks)
+k_stag_fx4(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, const void* lfx,
+           const void* links64) {
+    const SysBlock q = sys_block(npass, act);
+    if (!q.ok) return;
+    const PassDesc d = descs[q.j];
+    if (gated_off(e, d)) return;
+    const double alpha = (KIND == PASS_B || KIND == PASS_BC) ? e.sys[d.sys].alpha : 0.0;
+    double local = 0;
+    const int nh = vlen(g), per = blockDim.x >> 2;
+    for (int h0 = q.bx * per; h0 < nh; h0 += q.gx * per) {
+        const int h = h0 + (threadIdx.x >> 2);
+        const bool on = h < nh;
+        local += stag_site_fx4<NC, KIND, TO, false>(d, g, lfx, links64, alpha, pass_site<KIND == PASS_A>(on ? h : 0, g), on);
+    }
+    if (d.row >= 0) {
+        double tot;
+        if (reduce_last_n(e, d.row, local, tot, q.gx, q.bx)) finalize<KIND == PASS_BC>(e, d, tot);
+    }
+}
+
 static int device_sms() {
     static const int n = [] {
         int dev = 0, sms = 0;
@@ -133,9 +163,19 @@ static void launch_one(const Engine& e, const PassDesc* descs, StagGeom g, const
 template <int NC, int KIND, class TO>
 static void launch_fx(const Engine& e, const PassDesc* descs, const OpDev& op, int npass, const int* act, bool per,
                       cudaStream_t st) {
-    auto k = k_stag_fx<NC, KIND, TO>;
     const int64_t V = vlen(op.g);
     const int np = std::max(npass, 1);
+    if (V * np <= kFx4Sites) {
+        auto k4 = k_stag_fx4<NC, KIND, TO>;
+        int nt = kFx4Threads;
+        while (nt > 32 && (4 * V * np + nt - 1) / nt < 2 * device_sms()) nt >>= 1;
+        const int64_t need = (4 * V + nt - 1) / nt, res = resident_blocks((const void*)k4, nt);
+        const dim3 grid = (per && npass > 1) ? dim3((unsigned)npass, (unsigned)std::min(need, res))
+                                             : dim3((unsigned)std::max<int64_t>(np, std::min(need * np, res)));
+        k4<<<grid, nt, 0, st>>>(e, descs, npass, act, op.g, op.linksfx, op.links64);
+        return;
+    }
+    auto k = k_stag_fx<NC, KIND, TO>;
     int nt = kFxThreads;
     while (nt > 32 && ((V + nt - 1) / nt) * np < 2 * device_sms()) nt >>= 1;
     const int64_t need = (V + nt - 1) / nt, res = resident_blocks((const void*)k, nt);

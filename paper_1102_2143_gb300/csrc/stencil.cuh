@@ -271,6 +271,47 @@ __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* link
 template <class T, int KIND>
 using SiteAcc = typename std::conditional<(sizeof(T) == 4 && KIND != PASS_C), float, double>::type;
 
+// The epilogue KIND of a D pass at colour a of vector site x, y = (D src)_a
+// there; adds to the site's share of the reduction (nothing when d.row < 0).
+template <class T, int NC, int KIND, class TO, bool PL>
+__device__ __forceinline__ void stag_colour(const PassDesc& d, int x, int a, int V, T2<T> y, T alpha,
+                                            SiteAcc<T, KIND>& loc) {
+    const T2<T>* __restrict__ aux = (const T2<T>*)d.aux;
+    const T dd = (T)d.d;
+    const size_t i = vix<T, PL, NC>(x, a, V);
+    if (KIND == PASS_A) {
+        ((T2<T>*)d.out)[i] = y;
+        if (d.row >= 0) {
+            const T2<T> pa = aux[i];
+            loc += dd * (pa.x * pa.x + pa.y * pa.y) + y.x * y.x + y.y * y.y;
+        }
+    } else if (KIND == PASS_B || KIND == PASS_BC) {
+        T2<T>* r = (T2<T>*)d.out;
+        const T2<T> pa = aux[i];
+        const T2<T> ap = {dd * pa.x - y.x, dd * pa.y - y.y};
+        T2<T> ra = r[i];
+        ra.x -= alpha * ap.x;
+        ra.y -= alpha * ap.y;
+        r[i] = ra;
+        loc += ra.x * ra.x + ra.y * ra.y;
+    } else if (KIND == PASS_C) {
+        TO* out = (TO*)d.out;
+        const T2<T> xa = aux[i];
+        const double2 ba = d.b[(size_t)x * NC + a];
+        const double vx = ba.x - ((double)dd * xa.x - y.x);
+        const double vy = ba.y - ((double)dd * xa.y - y.y);
+        if (out) {
+            const size_t o = vix<TO, PL, NC>(x, a, V);
+            out[2 * o] = (TO)vx;
+            out[2 * o + 1] = (TO)vy;
+        }
+        loc += vx * vx + vy * vy;
+    } else {
+        const T2<T> xa = aux[i];
+        ((T2<T>*)d.out)[i] = {dd * xa.x - y.x, dd * xa.y - y.y};
+    }
+}
+
 // RECON = kLinksFx (FP64 only): `links` holds fixed-point limbs and links64
 // the FP64 links.
 constexpr int kLinksFx = 2;
@@ -278,65 +319,101 @@ template <class T, int NC, int RECON, int KIND, class TO, bool PL = false, bool 
 __device__ __forceinline__ SiteAcc<T, KIND> stag_site(const PassDesc& d, const StagGeom& g, const void* links,
                                             T alpha, int x, const void* links64 = nullptr) {
     const T2<T>* __restrict__ src = (const T2<T>*)d.src;
-    const T2<T>* __restrict__ aux = (const T2<T>*)d.aux;
-    const T dd = (T)d.d;
     const int V = vlen(g);
     T2<T> y[NC];
     if constexpr (RECON == kLinksFx) dslash_site_fx<NC, FRESH>(links, links64, src, x, g, y);
     else dslash_site<T, NC, RECON, PL>(links, src, x, g, y);
     x = vsite(x, g);  // the site's index in the vectors
-    if (KIND == PASS_A) {
-        T2<T>* out = (T2<T>*)d.out;
-        T loc = T(0);
+    SiteAcc<T, KIND> loc = 0;
 #pragma unroll
-        for (int a = 0; a < NC; ++a) {
-            out[vix<T, PL, NC>(x, a, V)] = y[a];
-            if (d.row >= 0) {
-                const T2<T> pa = aux[vix<T, PL, NC>(x, a, V)];
-                loc += dd * (pa.x * pa.x + pa.y * pa.y) + y[a].x * y[a].x + y[a].y * y[a].y;
-            }
-        }
-        return (SiteAcc<T, KIND>)loc;
-    } else if (KIND == PASS_B || KIND == PASS_BC) {
-        T2<T>* r = (T2<T>*)d.out;
-        T loc = T(0);
+    for (int a = 0; a < NC; ++a) stag_colour<T, NC, KIND, TO, PL>(d, x, a, V, y[a], alpha, loc);
+    return loc;
+}
+
+// The FP64 pass at one site by four lanes (consecutive lanes of a warp, lane & 3
+// = the direction): each takes its direction's two hops, the entries' exponent
+// is the largest of the four lanes', and the integer sums add across them.
+// Lane a < NC then runs the epilogue of colour a. All lanes of the warp call it;
+// on = false for those without a site.
+template <int NC, int KIND, class TO, bool FRESH>
+__device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeom& g, const void* lfx,
+                                                const void* links64, double alpha, int x, bool on) {
+    const double2* __restrict__ src = (const double2*)d.src;
+    const int mu = threadIdx.x & 3;
+    const int q0 = gdiv(x, g, 0), q1 = gdiv(q0, g, 1), q2 = gdiv(q1, g, 2);
+    const int c0 = x - q0 * g.L[0], c1 = q0 - q1 * g.L[1], c2 = q1 - q2 * g.L[2];
+    const int L = g.L[mu];
+    const int c = mu == 0 ? c0 : mu == 1 ? c1 : mu == 2 ? c2 : q2;
+    const int stride = (mu > 0 ? g.L[0] : 1) * (mu > 1 ? g.L[1] : 1) * (mu > 2 ? g.L[2] : 1);
+    const int par = ((mu > 0 ? c0 : 0) + (mu > 1 ? c1 : 0) + (mu > 2 ? c2 : 0)) & 1;
+    const int xf = c == L - 1 ? x - (L - 1) * stride : x + stride;
+    const int xb = c == 0 ? x + (L - 1) * stride : x - stride;
+    double2 v[2][NC];
+    unsigned e = 0;
 #pragma unroll
-        for (int a = 0; a < NC; ++a) {
-            const T2<T> pa = aux[vix<T, PL, NC>(x, a, V)];
-            const T2<T> ap = {dd * pa.x - y[a].x, dd * pa.y - y[a].y};
-            T2<T> ra = r[vix<T, PL, NC>(x, a, V)];
-            ra.x -= alpha * ap.x;
-            ra.y -= alpha * ap.y;
-            r[vix<T, PL, NC>(x, a, V)] = ra;
-            loc += ra.x * ra.x + ra.y * ra.y;
+    for (int b = 0; b < NC; ++b) {
+        v[0][b] = v[1][b] = {0.0, 0.0};
+        if (on) {
+            const double2* vf = src + (size_t)vsite(xf, g) * NC + b;
+            const double2* vb = src + (size_t)vsite(xb, g) * NC + b;
+            v[0][b] = FRESH ? *vf : __ldg(vf);
+            v[1][b] = FRESH ? *vb : __ldg(vb);
         }
-        return (SiteAcc<T, KIND>)loc;
-    } else if (KIND == PASS_C) {
-        TO* out = (TO*)d.out;
-        double loc = 0.0;
-#pragma unroll
-        for (int a = 0; a < NC; ++a) {
-            const T2<T> xa = aux[vix<T, PL, NC>(x, a, V)];
-            const double2 ba = d.b[(size_t)x * NC + a];
-            const double vx = ba.x - ((double)dd * xa.x - y[a].x);
-            const double vy = ba.y - ((double)dd * xa.y - y[a].y);
-            if (out) {
-                const size_t o = vix<TO, PL, NC>(x, a, V);
-                out[2 * o] = (TO)vx;
-                out[2 * o + 1] = (TO)vy;
-            }
-            loc += vx * vx + vy * vy;
-        }
-        return loc;
-    } else {
-        T2<T>* out = (T2<T>*)d.out;
-#pragma unroll
-        for (int a = 0; a < NC; ++a) {
-            const T2<T> xa = aux[vix<T, PL, NC>(x, a, V)];
-            out[vix<T, PL, NC>(x, a, V)] = {dd * xa.x - y[a].x, dd * xa.y - y[a].y};
-        }
-        return SiteAcc<T, KIND>(0);
+        fx_bound(e, v[0][b]);
+        fx_bound(e, v[1][b]);
     }
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+    const unsigned field = fx_field(e);
+    FxSum re[NC], im[NC];
+#pragma unroll
+    for (int a = 0; a < NC; ++a) re[a] = im[a] = {0, 0};
+    if (on) {
+#pragma unroll
+        for (int dir = 0; dir < 2; ++dir) {
+            const bool fwd = dir == 0;
+            const int4* __restrict__ U = (const int4*)lfx + fx_link<NC>(mu, fwd ? x : xb, g.V);
+            const int flip = fwd ? -par : par - 1;
+#pragma unroll
+            for (int b = 0; b < NC; ++b) {
+                int rh, rl, ih, il;
+                fx_split(v[dir][b].x, field, flip, rh, rl);
+                fx_split(v[dir][b].y, field, flip, ih, il);
+                const int zh = fwd ? -ih : ih, zl = fwd ? -il : il;
+                const int wh = fwd ? rh : -rh, wl = fwd ? rl : -rl;
+#pragma unroll
+                for (int a = 0; a < NC; ++a) {
+                    const int4 u = __ldg(U + (fwd ? a * NC + b : b * NC + a) * 32);
+                    fx_mac(re[a], u.x, u.y, rh, rl);
+                    fx_mac(im[a], u.x, u.y, ih, il);
+                    fx_mac(re[a], u.z, u.w, zh, zl);
+                    fx_mac(im[a], u.z, u.w, wh, wl);
+                }
+            }
+        }
+    }
+    // this lane's colour of the sum over the four directions
+    long long sr = 0, si = 0;
+#pragma unroll
+    for (int a = 0; a < NC; ++a) {
+        long long r = re[a].h + ((re[a].m + (1 << 27)) >> 28), i = im[a].h + ((im[a].m + (1 << 27)) >> 28);
+        r += __shfl_xor_sync(0xffffffffu, r, 1);
+        i += __shfl_xor_sync(0xffffffffu, i, 1);
+        r += __shfl_xor_sync(0xffffffffu, r, 2);
+        i += __shfl_xor_sync(0xffffffffu, i, 2);
+        if (a == mu) { sr = r; si = i; }
+    }
+    if (!on || mu >= NC) return 0.0;
+    double2 y = {fx_double(sr, field, 1), fx_double(si, field, 1)};
+    if (!fx_in_range(field)) {
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
+#pragma unroll
+        for (int a = 0; a < NC; ++a)
+            if (a == mu) y = r.y[a];
+    }
+    double loc = 0.0;
+    stag_colour<double, NC, KIND, TO, true>(d, vsite(x, g), mu, vlen(g), y, alpha, loc);
+    return loc;
 }
 
 }  // namespace msc
