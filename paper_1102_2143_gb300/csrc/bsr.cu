@@ -147,10 +147,11 @@ template <int BD> constexpr int kFxRowGroup = BD == 3 ? 3 : 4;
 // FX (FP64, bd > 1): rows by fixed-point sums (bsr_row_fx), 128-thread blocks.
 template <class T, int BD, int KIND, class TO, bool FX = false>
 __global__ void __launch_bounds__(FX ? kFxRowThreads : kThreads, FX ? kFxRowBlocks : sizeof(T) == 4 ? 4 : 3)
-k_bsr(Engine e, const PassDesc* descs, int npass, const int* act, OpDev A, const T2<T>* __restrict__ vals) {
+k_bsr(Engine e, const PassDesc* descs, int npass, const int* act, OpDev A, const T2<T>* __restrict__ vals,
+      PassDesc one) {
     const SysBlock q = sys_block(npass, act);
     if (!q.ok) return;
-    const PassDesc d = descs[q.j];
+    const PassDesc d = descs ? descs[q.j] : one;
     if (gated_off(e, d)) return;
     const T2<T>* __restrict__ src = (const T2<T>*)d.src;
     const T2<T>* __restrict__ aux = (const T2<T>*)d.aux;
@@ -374,30 +375,30 @@ template <class T, int BD, int KIND, class TO>
 static void launch_one(const Engine& e, const PassDesc* descs, const OpDev& A, const T2<T>* vals,
                        int npass, const int* act, bool per, cudaStream_t st) {
     auto k = k_bsr<T, BD, KIND, TO>;
-    k<<<multi_grid((const void*)k, A.nbr, npass, per), kThreads, 0, st>>>(e, descs, npass, act, A, vals);
+    k<<<multi_grid((const void*)k, A.nbr, npass, per), kThreads, 0, st>>>(e, descs, npass, act, A, vals, PassDesc{});
 }
 
 template <int BD, int KIND, class TO>
 static void launch_one_fx(const Engine& e, const PassDesc* descs, const OpDev& A, int npass, const int* act, bool per,
-                          cudaStream_t st) {
+                          const PassDesc& one, cudaStream_t st) {
     auto k = k_bsr<double, BD, KIND, TO, true>;
     const int64_t np = std::max(npass, 1), need = (A.nbr + kFxRowThreads - 1) / kFxRowThreads;
     const int64_t res = resident_blocks((const void*)k, kFxRowThreads);
     const dim3 grid = (per && npass > 1) ? dim3((unsigned)np, (unsigned)std::min(need, res))
                                          : dim3((unsigned)std::max(np, std::min(need * np, res)));
-    k<<<grid, kFxRowThreads, 0, st>>>(e, descs, npass, act, A, nullptr);
+    k<<<grid, kFxRowThreads, 0, st>>>(e, descs, npass, act, A, nullptr, one);
 }
 
 template <int BD>
 static cudaError_t launch_bd_fx(int kind, int out_f32, const Engine& e, const PassDesc* descs, const OpDev& A,
-                                int npass, const int* act, bool per, cudaStream_t st) {
+                                int npass, const int* act, bool per, const PassDesc& one, cudaStream_t st) {
     switch (kind) {
-        case PASS_A: launch_one_fx<BD, PASS_A, double>(e, descs, A, npass, act, per, st); break;
+        case PASS_A: launch_one_fx<BD, PASS_A, double>(e, descs, A, npass, act, per, one, st); break;
         case PASS_C:
-            if (out_f32) launch_one_fx<BD, PASS_C, float>(e, descs, A, npass, act, per, st);
-            else launch_one_fx<BD, PASS_C, double>(e, descs, A, npass, act, per, st);
+            if (out_f32) launch_one_fx<BD, PASS_C, float>(e, descs, A, npass, act, per, one, st);
+            else launch_one_fx<BD, PASS_C, double>(e, descs, A, npass, act, per, one, st);
             break;
-        case PASS_D: launch_one_fx<BD, PASS_D, double>(e, descs, A, npass, act, per, st); break;
+        case PASS_D: launch_one_fx<BD, PASS_D, double>(e, descs, A, npass, act, per, one, st); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -464,9 +465,11 @@ cudaError_t launch_bsr_pass(const OpDev& op, int prec, int kind, int out_f32, co
         return launch_bsr_multi(op, e, d_descs, npass, act, kMultiGroup,
                                 (npass + kMultiGroup - 1) / kMultiGroup, st);
     if (prec == PREC_F64 && op.valsfx) {
-        if (op.bd == 2) return launch_bd_fx<2>(kind, out_f32, e, d_descs, op, npass, act, per, st);
-        return launch_bd_fx<3>(kind, out_f32, e, d_descs, op, npass, act, per, st);
+        const PassDesc one = d_descs ? PassDesc{} : *h_desc;  // no device descriptor: the host's, as a parameter
+        if (op.bd == 2) return launch_bd_fx<2>(kind, out_f32, e, d_descs, op, npass, act, per, one, st);
+        return launch_bd_fx<3>(kind, out_f32, e, d_descs, op, npass, act, per, one, st);
     }
+    if (!d_descs) return cudaErrorInvalidValue;
     if (prec == PREC_F64) {
         switch (op.bd) {
             case 1: return launch_bd<double, 1>(kind, out_f32, e, d_descs, op, op.vals64, npass, act, per, st);

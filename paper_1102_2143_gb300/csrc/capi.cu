@@ -1065,6 +1065,61 @@ int msc_staggered_export_bsr(msc_ctx* c, const msc_op* op, int64_t* row_ptr, int
     return e == cudaSuccess ? MSC_OK : cuda_status(e);
 }
 
+// Whether the FP64 kernels can read or write [n] complex at p themselves:
+// memory of this device (not managed, not a peer's) on a 16-byte boundary.
+static bool kernel_ready(const void* p, int device) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device && ((uintptr_t)p & 15) == 0;
+}
+
+// FP64 applies on the fixed-point kernels: the passes' descriptors are kernel
+// parameters and the caller's vectors are used in place where the kernels can
+// (a staged copy of a 4^4 to 24^4 vector and the two descriptor uploads took
+// as long as the passes: A x at 10 x 6 x 14 x 18 47 us a call against 28).
+// Input and output may be the same vector of a staggered A x (its second
+// pass reads the input at the output's own site only); other overlaps are
+// staged.
+static int apply_direct(msc_ctx* c, const OpDev& A, double sigma, const double* in, double* out, bool dslash) {
+    const int64_t n = A.n, npad = (n + 63) / 64 * 64;
+    const int ws = ensure_ws(c, npad, 3, 1, 1, 16);
+    if (ws) return ws;
+    double2* t64 = (double2*)c->t64.p;
+    const double2* src = (const double2*)in;
+    double2* dst = (double2*)out;
+    const bool stag = A.kind == OP_STAGGERED;
+    const bool apart = in + 2 * n <= out || out + 2 * n <= in;
+    const bool same_ok = stag && !dslash && (const double*)out == in;
+    if (!kernel_ready(in, c->device) || !(apart || same_ok)) {
+        CK(cudaMemcpyAsync(t64, in, n * 16, cudaMemcpyDefault, c->work));
+        src = t64;
+    }
+    const bool direct_out = kernel_ready(out, c->device);
+    if (!direct_out) dst = t64 + 2 * npad;
+    double2* mid = t64 + npad;
+    const Engine none{};
+    if (stag) {
+        const PassDesc d1 = mkdesc(src, nullptr, nullptr, dslash ? dst : mid, 0.0, -1, -1, FIN_NONE);
+        CK(launch_stag_pass(A, PREC_F64, PASS_A, 0, none, nullptr, 1, c->work, nullptr, false, &d1));
+        c->launches++;
+        if (!dslash) {
+            const PassDesc d2 = mkdesc(mid, src, nullptr, dst, A.mass * A.mass + sigma, -1, -1, FIN_NONE);
+            CK(launch_stag_pass(A, PREC_F64, PASS_D, 0, none, nullptr, 1, c->work, nullptr, false, &d2));
+            c->launches++;
+        }
+    } else {
+        const PassDesc d = mkdesc(src, src, nullptr, dst, sigma, -1, -1, FIN_NONE);
+        CK(launch_bsr_pass(A, PREC_F64, PASS_D, 0, none, nullptr, 1, c->work, nullptr, false, &d));
+        c->launches++;
+    }
+    if (!direct_out) CK(cudaMemcpyAsync(out, dst, n * 16, cudaMemcpyDefault, c->work));
+    CK(cudaStreamSynchronize(c->work));
+    return MSC_OK;
+}
+
 // out = (A + sigma) in (or D in when dslash) through the operator kernels.
 static int apply_impl(msc_ctx* c, const msc_op* op, double sigma, const double* in, double* out,
                       int precision, bool dslash) {
@@ -1074,6 +1129,8 @@ static int apply_impl(msc_ctx* c, const msc_op* op, double sigma, const double* 
     int st = begin(c);
     if (st) return st;
     const OpDev& A = op->dev;
+    if (precision == MSC_FP64 && (A.kind == OP_STAGGERED ? (void*)A.linksfx : (void*)A.valsfx))
+        return apply_direct(c, A, sigma, in, out, dslash);
     const int64_t n = A.n, npad = (n + 63) / 64 * 64;
     st = ensure_ws(c, npad, 3, 1, 1, 16);
     if (st) return st;
@@ -2538,11 +2595,17 @@ extern "C" int msc_op_apply_noalloc(const msc_op* op, double sigma, const double
         double2* t = (double2*)((char*)base + kNoallocDescBytes);
         const PassDesc d1 = mkdesc(in, nullptr, nullptr, t, 0.0, -1, -1, FIN_NONE);
         const PassDesc d2 = mkdesc(t, in, nullptr, out, A.mass * A.mass + sigma, -1, -1, FIN_NONE);
-        k_noalloc_store_descs<<<1, 32, 0, st>>>(descs, d1, d2);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = cudaSuccess;
         Engine none{};
-        if (e == cudaSuccess) e = launch_stag_pass(A, PREC_F64, PASS_A, 0, none, descs, 1, st);
-        if (e == cudaSuccess) e = launch_stag_pass(A, PREC_F64, PASS_D, 0, none, descs + 1, 1, st);
+        const bool fx = A.linksfx != nullptr;  // its kernels take the descriptors as parameters
+        if (!fx) {
+            k_noalloc_store_descs<<<1, 32, 0, st>>>(descs, d1, d2);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess)
+            e = launch_stag_pass(A, PREC_F64, PASS_A, 0, none, descs, 1, st, nullptr, false, fx ? &d1 : nullptr);
+        if (e == cudaSuccess)
+            e = launch_stag_pass(A, PREC_F64, PASS_D, 0, none, descs + 1, 1, st, nullptr, false, fx ? &d2 : nullptr);
         if (e != cudaSuccess) status = cuda_status(e);
     }
     if (prev != dev) cudaSetDevice(prev);

@@ -71,9 +71,11 @@ struct OpDev {
 // `act` (device, optional): {count, indices} of the passes to run (see
 // sys_block in common.cuh); null runs all npass.
 // per_system: one whole grid row per pass (see sys_block).
+// one (host, optional; FP64 on linksfx only): the single pass, as a kernel
+// parameter instead of a device descriptor.
 cudaError_t launch_stag_pass(const OpDev& op, int prec, int kind, int out_f32, const Engine& e,
                              const PassDesc* d_descs, int npass, cudaStream_t st, const int* act = nullptr,
-                             bool per_system = false);
+                             bool per_system = false, const PassDesc* one = nullptr);
 // FP32 staggered passes of several systems sharing the operator, the links
 // loaded once per group of systems (PASS_A and PASS_B of a solve stage;
 // every descriptor has a reduction row; FP32 vectors colour-planar). `act`
@@ -94,6 +96,8 @@ cudaError_t launch_stag_tile(const OpDev& op, int kind, const Engine& e, const P
 // h_desc (optional): host copy of the single pass's descriptor; a one-system
 // FP32 PASS_A then takes its source and output pointers from it as kernel
 // parameters (the device descriptor must hold the same pointers).
+// With d_descs null (FP64 on valsfx only) the kernel takes the whole
+// descriptor from it.
 cudaError_t launch_bsr_pass(const OpDev& op, int prec, int kind, int out_f32, const Engine& e,
                             const PassDesc* d_descs, int npass, cudaStream_t st, const int* act = nullptr,
                             bool per_system = false, const PassDesc* h_desc = nullptr);

@@ -69,6 +69,7 @@ k_stag(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, c
     }
 }
 
+// (descs null: the single pass `one`, a kernel parameter.)
 // The FP64 pass over unitary links by fixed-point sums (dslash_site_fx; links
 // that are not unitary may have any range and keep k_stag<double>). Four
 // 128-thread blocks per SM at 128 registers: three at 168 take 2% longer and
@@ -80,10 +81,10 @@ constexpr int kFxThreads = 128, kFxBlocks = 4;
 template <int NC, int KIND, class TO>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocks)
 k_stag_fx(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, const void* lfx,
-          const void* links64) {
+          const void* links64, PassDesc one) {
     const SysBlock q = sys_block(npass, act);
     if (!q.ok) return;
-    const PassDesc d = descs[q.j];
+    const PassDesc d = descs ? descs[q.j] : one;
     if (gated_off(e, d)) return;
     const double alpha = (KIND == PASS_B || KIND == PASS_BC) ? e.sys[d.sys].alpha : 0.0;
     double local = 0;
@@ -108,10 +109,10 @@ constexpr int64_t kFx4Sites = 24576;
 template <int NC, int KIND, class TO>
 __global__ void __launch_bounds__(kFx4Threads, kFxBlocks)
 k_stag_fx4(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, const void* lfx,
-           const void* links64) {
+           const void* links64, PassDesc one) {
     const SysBlock q = sys_block(npass, act);
     if (!q.ok) return;
-    const PassDesc d = descs[q.j];
+    const PassDesc d = descs ? descs[q.j] : one;
     if (gated_off(e, d)) return;
     const double alpha = (KIND == PASS_B || KIND == PASS_BC) ? e.sys[d.sys].alpha : 0.0;
     double local = 0;
@@ -162,7 +163,7 @@ static void launch_one(const Engine& e, const PassDesc* descs, StagGeom g, const
 
 template <int NC, int KIND, class TO>
 static void launch_fx(const Engine& e, const PassDesc* descs, const OpDev& op, int npass, const int* act, bool per,
-                      cudaStream_t st) {
+                      const PassDesc& one, cudaStream_t st) {
     const int64_t V = vlen(op.g);
     const int np = std::max(npass, 1);
     if (V * np <= kFx4Sites) {
@@ -172,7 +173,7 @@ static void launch_fx(const Engine& e, const PassDesc* descs, const OpDev& op, i
         const int64_t need = (4 * V + nt - 1) / nt, res = resident_blocks((const void*)k4, nt);
         const dim3 grid = (per && npass > 1) ? dim3((unsigned)npass, (unsigned)std::min(need, res))
                                              : dim3((unsigned)std::max<int64_t>(np, std::min(need * np, res)));
-        k4<<<grid, nt, 0, st>>>(e, descs, npass, act, op.g, op.linksfx, op.links64);
+        k4<<<grid, nt, 0, st>>>(e, descs, npass, act, op.g, op.linksfx, op.links64, one);
         return;
     }
     auto k = k_stag_fx<NC, KIND, TO>;
@@ -181,23 +182,23 @@ static void launch_fx(const Engine& e, const PassDesc* descs, const OpDev& op, i
     const int64_t need = (V + nt - 1) / nt, res = resident_blocks((const void*)k, nt);
     const dim3 grid = (per && npass > 1) ? dim3((unsigned)npass, (unsigned)std::min(need, res))
                                          : dim3((unsigned)std::max<int64_t>(np, std::min(need * np, res)));
-    k<<<grid, nt, 0, st>>>(e, descs, npass, act, op.g, op.linksfx, op.links64);
+    k<<<grid, nt, 0, st>>>(e, descs, npass, act, op.g, op.linksfx, op.links64, one);
 }
 
 template <int NC>
 static cudaError_t launch_kind_fx(int kind, int out_f32, const Engine& e, const PassDesc* descs, const OpDev& op,
-                                  int npass, const int* act, bool per, cudaStream_t st) {
+                                  int npass, const int* act, bool per, const PassDesc& one, cudaStream_t st) {
     switch (kind) {
-        case PASS_A: launch_fx<NC, PASS_A, double>(e, descs, op, npass, act, per, st); break;
+        case PASS_A: launch_fx<NC, PASS_A, double>(e, descs, op, npass, act, per, one, st); break;
         case PASS_B:
-            if (e.cond_flag) launch_fx<NC, PASS_BC, double>(e, descs, op, npass, act, per, st);
-            else launch_fx<NC, PASS_B, double>(e, descs, op, npass, act, per, st);
+            if (e.cond_flag) launch_fx<NC, PASS_BC, double>(e, descs, op, npass, act, per, one, st);
+            else launch_fx<NC, PASS_B, double>(e, descs, op, npass, act, per, one, st);
             break;
         case PASS_C:
-            if (out_f32) launch_fx<NC, PASS_C, float>(e, descs, op, npass, act, per, st);
-            else launch_fx<NC, PASS_C, double>(e, descs, op, npass, act, per, st);
+            if (out_f32) launch_fx<NC, PASS_C, float>(e, descs, op, npass, act, per, one, st);
+            else launch_fx<NC, PASS_C, double>(e, descs, op, npass, act, per, one, st);
             break;
-        default: launch_fx<NC, PASS_D, double>(e, descs, op, npass, act, per, st); break;
+        default: launch_fx<NC, PASS_D, double>(e, descs, op, npass, act, per, one, st); break;
     }
     return cudaGetLastError();
 }
@@ -222,11 +223,15 @@ static cudaError_t launch_kind(int kind, int out_f32, const Engine& e, const Pas
 }
 
 cudaError_t launch_stag_pass(const OpDev& op, int prec, int kind, int out_f32, const Engine& e,
-                             const PassDesc* d_descs, int npass, cudaStream_t st, const int* act, bool per) {
+                             const PassDesc* d_descs, int npass, cudaStream_t st, const int* act, bool per,
+                             const PassDesc* one) {
     if (prec == PREC_F64 && op.linksfx) {
-        if (op.nc == 3) return launch_kind_fx<3>(kind, out_f32, e, d_descs, op, npass, act, per, st);
-        return launch_kind_fx<2>(kind, out_f32, e, d_descs, op, npass, act, per, st);
+        const PassDesc h = one ? *one : PassDesc{};
+        if (one) d_descs = nullptr;
+        if (op.nc == 3) return launch_kind_fx<3>(kind, out_f32, e, d_descs, op, npass, act, per, h, st);
+        return launch_kind_fx<2>(kind, out_f32, e, d_descs, op, npass, act, per, h, st);
     }
+    if (one) return cudaErrorInvalidValue;
     if (prec == PREC_F64) {
         if (op.nc == 3) return launch_kind<double, 3, 0>(kind, out_f32, e, d_descs, op.g, op.links64, npass, act, per, st);
         return launch_kind<double, 2, 0>(kind, out_f32, e, d_descs, op.g, op.links64, npass, act, per, st);

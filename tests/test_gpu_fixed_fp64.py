@@ -197,3 +197,45 @@ def test_bsr_out_of_range_takes_fp64(ctx, bd):
     b[3, 0, 0] = np.inf
     out, want = apply(b, v), oracle.bsr_apply(rp, ci, b, v)
     assert np.array_equal(np.isfinite(out), np.isfinite(want))
+
+
+@pytest.mark.parametrize("bsr", [False, True])
+def test_apply_in_place_overlapping_and_unaligned(ctx, bsr):
+    """msc_op_apply on the caller's vectors in place: the same results whether
+    input and output are the same vector, overlap by part, start between
+    16-byte boundaries, or lie on the host. Exact: the kernels are the same."""
+    dims, nc = (4, 6, 2, 4), 3
+    U = inputs.su_n_links(dims, nc, 0.9, 95)
+    op = msc.msc_op_staggered(ctx, nc, dims, torch.from_numpy(U).cuda(), 0.1)
+    if bsr:
+        nbr, nnzb, bd = msc.msc_op_bsr_size(op)
+        rp = torch.empty(nbr + 1, dtype=torch.int64, device="cuda")
+        ci = torch.empty(nnzb, dtype=torch.int32, device="cuda")
+        va = torch.empty((nnzb, bd, bd), dtype=torch.complex128, device="cuda")
+        msc.msc_staggered_export_bsr(ctx, op, rp, ci, va)
+        op = msc.msc_op_bsr(ctx, nbr, bd, rp, ci, va)
+    n = inputs.volume(dims) * nc
+    v = inputs.gaussian_source(n, 96)
+    x = torch.from_numpy(v).cuda()
+    want = torch.empty_like(x)
+    msc.msc_op_apply(ctx, op, 0.2, x, want, msc.MSC_FP64)
+    assert torch.equal(x, torch.from_numpy(v).cuda())
+    host = np.empty_like(v)
+    msc.msc_op_apply(ctx, op, 0.2, v, host, msc.MSC_FP64)
+    assert np.array_equal(host, want.cpu().numpy())
+    same = x.clone()
+    msc.msc_op_apply(ctx, op, 0.2, same, same, msc.MSC_FP64)
+    assert torch.equal(same, want)
+    buf = torch.zeros(2 * (n + 64), dtype=torch.float64, device="cuda")
+    for at_in, at_out in ((0, 34), (34, 0), (1, 1), (3, 0), (0, 5)):
+        i = buf[at_in:at_in + 2 * n]
+        i.copy_(torch.view_as_real(x).reshape(-1))
+        base = buf.data_ptr()
+        msc.msc_op_apply(ctx, op, 0.2, base + 8 * at_in, base + 8 * at_out, msc.MSC_FP64)
+        assert torch.equal(buf[at_out:at_out + 2 * n], torch.view_as_real(want).reshape(-1)), (at_in, at_out)
+    if not bsr:
+        d = torch.empty_like(x)
+        msc.msc_op_dslash(ctx, op, x, d)
+        y = x.clone()
+        msc.msc_op_dslash(ctx, op, y, y)
+        assert torch.equal(y, d)
