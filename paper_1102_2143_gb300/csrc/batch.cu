@@ -28,52 +28,85 @@ __device__ __forceinline__ int find_system(const int* __restrict__ map, int J, i
     return lo;
 }
 
-struct VBlock {
-    int j;   // system
-    int lb;  // block within the system
-    int nb;  // blocks of the system
-};
-
-__device__ __forceinline__ VBlock vblock(const BTab& t, const int* map, int vb) {
+// The virtual blocks of the three maps, one entry each, written once per set
+// of active systems: searching the map in every block was a chain of six or
+// seven dependent loads (3,000 clocks) before the block's first vector load.
+__global__ void kb_expand(BTab t, VBlock* vsite, VBlock* vvec, VBlock* vupd) {
     const int J = __ldg(t.hdr);
-    const int k = find_system(map, J, vb);
-    const int b0 = __ldg(map + k);
-    VBlock v;
-    v.j = __ldg(t.act + k);
-    v.lb = vb - b0;
-    v.nb = __ldg(map + k + 1) - b0;
-    return v;
+    for (int m = 0; m < 3; ++m) {
+        const int* map = m == 0 ? t.msite : m == 1 ? t.mvec : t.mupd;
+        VBlock* out = m == 0 ? vsite : m == 1 ? vvec : vupd;
+        const int total = __ldg(t.hdr + 1 + m);
+        for (int vb = blockIdx.x * blockDim.x + threadIdx.x; vb < total; vb += gridDim.x * blockDim.x) {
+            const int k = find_system(map, J, vb), b0 = __ldg(map + k), j = __ldg(t.act + k);
+            out[vb] = {j, vb - b0, __ldg(map + k + 1) - b0, t.sys[j].op};
+        }
+    }
 }
 
+cudaError_t launch_b_expand(const BTab& t, VBlock* vsite, VBlock* vvec, VBlock* vupd, int blocks, cudaStream_t st) {
+    kb_expand<<<std::max(1, std::min((blocks + 255) / 256, 1024)), 256, 0, st>>>(t, vsite, vvec, vupd);
+    return cudaGetLastError();
+}
+
+__device__ __forceinline__ VBlock vblock(const VBlock* table, int vb) {
+    const int4 e = __ldg((const int4*)table + vb);
+    return {e.x, e.y, e.z, e.w};
+}
+
+// FP32: a block walks a run of consecutive virtual blocks and reduces once per
+// system of the run, not once per virtual block (the sum and the arrival's
+// round trip held the block's other warps at its barrier for a quarter of the
+// pass): a system is summed over the blocks whose runs meet it, block_of(first)
+// to block_of(last). (16 problems x 4 sources: 46 -> 38 and 56 -> 50 us a
+// pass.) FP64 passes are mostly reliable updates, in which a few systems of the
+// batch take part: their virtual blocks are dealt over all blocks instead (as
+// runs 200 us, as single ones 60-70).
+// FP32 at four 256-thread blocks' registers per SM, FP64 at two: three / one
+// take 1% / 6% longer, two in FP32 13%.
 template <class T, int KIND, class TO>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) kb_stag(Engine e, const PassDesc* descs, BTab t) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) kb_stag(Engine e, const PassDesc* descs, BTab t) {
     const int total = __ldg(t.hdr + 1);
-    for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        const VBlock q = vblock(t, t.msite, vb);
+    const int grid = min((int)gridDim.x, total), b = blockIdx.x;
+    if (b >= grid) return;
+    // block b's run is [b total / grid, (b + 1) total / grid)
+    auto block_of = [&](int vb) { return (int)((((long long)vb + 1) * grid - 1) / total); };
+    constexpr bool kRuns = sizeof(T) == 4;
+    const int first = kRuns ? (int)((long long)b * total / grid) : b;
+    const int last = kRuns ? (int)((long long)(b + 1) * total / grid) : total;
+    double local = 0.0;
+    for (int vb = first; vb < last; vb += kRuns ? 1 : grid) {
+        const VBlock q = vblock(t.vsite, vb);
+        // the system of a batch's pass is its gating system: everything is
+        // loaded by q alone, side by side
         const PassDesc d = descs[q.j];
-        if (gated_off(e, d)) continue;
-        const BOp op = t.ops[t.sys[q.j].op];
-        const T alpha = (KIND == PASS_B || KIND == PASS_BC) ? (T)e.sys[d.sys].alpha : T(0);
-        double local = 0.0;
+        const BOp op = t.ops[q.op];
+        const int st = load_status(&e.sys[q.j]), ru = __ldcg(&e.sys[q.j].ru);
+        const T alpha = (KIND == PASS_B || KIND == PASS_BC) ? (T)e.sys[q.j].alpha : T(0);
+        if (st != ST_RUNNING || (d.gate == 1 && ru == 0)) continue;
         const int x = q.lb * blockDim.x + threadIdx.x;
         if (x < op.g.V) {
             if constexpr (sizeof(T) == 4) {
                 if (op.nc == 3) {
-                    if (op.recon) local = stag_site<T, 3, 1, KIND, TO>(d, op.g, op.l32, alpha, x);
-                    else local = stag_site<T, 3, 0, KIND, TO>(d, op.g, op.l32, alpha, x);
+                    if (op.recon) local += (double)stag_site<T, 3, 1, KIND, TO>(d, op.g, op.l32, alpha, x);
+                    else local += (double)stag_site<T, 3, 0, KIND, TO>(d, op.g, op.l32, alpha, x);
                 } else {
-                    if (op.recon) local = stag_site<T, 2, 1, KIND, TO>(d, op.g, op.l32, alpha, x);
-                    else local = stag_site<T, 2, 0, KIND, TO>(d, op.g, op.l32, alpha, x);
+                    if (op.recon) local += (double)stag_site<T, 2, 1, KIND, TO>(d, op.g, op.l32, alpha, x);
+                    else local += (double)stag_site<T, 2, 0, KIND, TO>(d, op.g, op.l32, alpha, x);
                 }
             } else {
-                if (op.nc == 3) local = stag_site<T, 3, kLinksFx, KIND, TO>(d, op.g, op.lfx, alpha, x, op.l64);
-                else local = stag_site<T, 2, kLinksFx, KIND, TO>(d, op.g, op.lfx, alpha, x, op.l64);
+                if (op.nc == 3) local += stag_site<T, 3, kLinksFx, KIND, TO>(d, op.g, op.lfx, alpha, x, op.l64);
+                else local += stag_site<T, 2, kLinksFx, KIND, TO>(d, op.g, op.lfx, alpha, x, op.l64);
             }
         }
+        if (kRuns && q.lb + 1 < q.nb && vb + 1 < last) continue;  // the run goes on in this system
         if (d.row >= 0) {
+            const int start = vb - q.lb, b0 = block_of(start);
+            const int count = kRuns ? block_of(start + q.nb - 1) - b0 + 1 : q.nb, mine = kRuns ? b - b0 : q.lb;
             double tot;
-            if (reduce_last_n(e, d.row, local, tot, q.nb, q.lb)) finalize<KIND == PASS_BC>(e, d, tot);
+            if (reduce_last_n(e, d.row, local, tot, count, mine)) finalize<KIND == PASS_BC>(e, d, tot);
         }
+        local = 0.0;
     }
 }
 
@@ -84,7 +117,7 @@ __global__ void __launch_bounds__(kThreads) kb_init(Engine e, BVec v, BTab t) {
     constexpr int cpu = U16<T>::cpu;
     const int total = __ldg(t.hdr + 2);
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        const VBlock w = vblock(t, t.mvec, vb);
+        const VBlock w = vblock(t.vvec, vb);
         const int j = w.j;
         const BSys q = t.sys[j];
         const SysScalars* s = &e.sys[j];
@@ -136,7 +169,7 @@ __global__ void __launch_bounds__(kThreads) kb_init_from_r(Engine e, BVec v, BTa
     const int total = __ldg(t.hdr + 2);
     const bool mixed = (void*)v.xit != (void*)v.x64;
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        const VBlock w = vblock(t, t.mvec, vb);
+        const VBlock w = vblock(t.vvec, vb);
         const int j = w.j;
         const SysScalars* s = &e.sys[j];
         if (load_status(s) != ST_RUNNING) continue;
@@ -169,7 +202,7 @@ __global__ void __launch_bounds__(kThreads) kb_update(Engine e, BVec v, BTab t) 
     __shared__ int sf[kMaxShifts];
     const int total = __ldg(t.hdr + 3);
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        const VBlock w = vblock(t, t.mupd, vb);
+        const VBlock w = vblock(t.vupd, vb);
         const int j = w.j;
         SysScalars* s = &e.sys[j];
         const int st = load_status(s);
@@ -250,7 +283,7 @@ __global__ void __launch_bounds__(kThreads) kb_update(Engine e, BVec v, BTab t) 
 __global__ void __launch_bounds__(kThreads) kb_fold(Engine e, BVec v, BTab t, int only_ru) {
     const int total = __ldg(t.hdr + 2);
     for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-        const VBlock w = vblock(t, t.mvec, vb);
+        const VBlock w = vblock(t.vvec, vb);
         const int j = w.j;
         const SysScalars* s = &e.sys[j];
         const int st = load_status(s);

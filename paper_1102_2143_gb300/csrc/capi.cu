@@ -76,6 +76,7 @@ struct msc_ctx {
     Buf sys, slot, partial, counter, out_red, descs;
     Buf b64, x64, t64, r, p, t, ps, xit;
     Buf coef, force;  // adjoint: weights c_s and a link-shaped output
+    Buf bvb;          // batched solves: virtual-block tables
     Buf btab;         // batched solves: system table, operator table, block maps
     Buf actb;         // {count, indices} of the systems still iterating (refinement)
     Buf bcg;          // BiCGStab-M scalars: one BcgSys, then S BcgSlot
@@ -762,7 +763,7 @@ int msc_destroy(msc_ctx* c) {
         if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
     Buf* bufs[] = {&c->sys, &c->slot, &c->partial, &c->counter, &c->out_red, &c->descs,
                    &c->b64, &c->x64, &c->t64, &c->r, &c->p, &c->t, &c->ps, &c->xit,
-                   &c->coef, &c->force, &c->btab, &c->actb, &c->condf, &c->bcg,
+                   &c->coef, &c->force, &c->btab, &c->bvb, &c->actb, &c->condf, &c->bcg,
                    &c->pb, &c->px0, &c->ptmp, &c->gbar, &c->errf};
     for (Buf* b : bufs)
         if (b->p) cudaFree(b->p);
@@ -1770,11 +1771,15 @@ static size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 // systems still iterating changes; kernels read them when they run.
 struct BatchHost {
     int cap = 0, nops = 0;
+    int64_t cap_site = 0, cap_vec = 0;  // entries of the virtual-block tables
     size_t off_ops = 0, off_hdr = 0, off_act = 0, off_ms = 0, off_mv = 0, off_mu = 0, total = 0;
     BTab tab{};
 };
 
-static int batch_layout(msc_ctx* c, int cap, int nops, BatchHost& bh) {
+// The smallest launch shapes (see autotune_batch): they bound the virtual blocks.
+constexpr int kMinSiteThreads = 64, kMinVecThreads = 128;
+
+static int batch_layout(msc_ctx* c, int cap, int nops, int64_t cap_site, int64_t cap_vec, BatchHost& bh) {
     bh.cap = cap;
     bh.nops = nops;
     bh.off_ops = al256(sizeof(BSys) * cap);
@@ -1784,8 +1789,11 @@ static int batch_layout(msc_ctx* c, int cap, int nops, BatchHost& bh) {
     bh.off_mv = bh.off_ms + al256(sizeof(int) * (cap + 1));
     bh.off_mu = bh.off_mv + al256(sizeof(int) * (cap + 1));
     bh.total = bh.off_mu + al256(sizeof(int) * (cap + 1));
+    bh.cap_site = cap_site;
+    bh.cap_vec = cap_vec;
     bool moved = false;
     CK(grow(c, c->btab, bh.total, moved));
+    CK(grow(c, c->bvb, sizeof(VBlock) * (size_t)(cap_site + 2 * cap_vec), moved));
     if (moved) c->gen++;
     if (c->h_act_cap < (int64_t)(bh.total / sizeof(int)) + 1) {
         if (c->h_act) cudaFreeHost(c->h_act);
@@ -1800,6 +1808,9 @@ static int batch_layout(msc_ctx* c, int cap, int nops, BatchHost& bh) {
     bh.tab.msite = (const int*)(base + bh.off_ms);
     bh.tab.mvec = (const int*)(base + bh.off_mv);
     bh.tab.mupd = (const int*)(base + bh.off_mu);
+    bh.tab.vsite = (const VBlock*)c->bvb.p;
+    bh.tab.vvec = bh.tab.vsite + cap_site;
+    bh.tab.vupd = bh.tab.vvec + cap_vec;
     return MSC_OK;
 }
 
@@ -1851,8 +1862,11 @@ static int set_active(msc_ctx* c, const BatchHost& bh, const std::vector<BSys>& 
     hdr[1] = (int)a;
     hdr[2] = (int)b;
     hdr[3] = (int)u;
+    if (a > bh.cap_site || b > bh.cap_vec || u > bh.cap_vec) return MSC_ERR_UNSUPPORTED;
     CK(cudaMemcpyAsync((char*)c->btab.p + bh.off_hdr, stage, bh.total - bh.off_hdr, cudaMemcpyHostToDevice,
                        c->work));
+    VBlock* vs = (VBlock*)c->bvb.p;
+    CK(launch_b_expand(bh.tab, vs, vs + bh.cap_site, vs + bh.cap_site + bh.cap_vec, (int)std::max(a, b), c->work));
     return MSC_OK;
 }
 
@@ -1961,13 +1975,13 @@ static cudaError_t build_chunk_graph_b_cond(msc_ctx* c, int prec, int chunk, con
 
 static int get_graph_b(msc_ctx* c, int prec, int chunk, bool reliable, const BTab& t, const BatchShape& sh,
                        GraphEntry** out) {
-    char key[200];
+    char key[256];
     // every table address is part of the key: their offsets depend on the
     // batch's capacity
-    snprintf(key, sizeof key, "batch|%d|%d|%d|%d|%d|%d|%p|%p|%p|%p|%p|%p|%p", prec, chunk, (int)reliable,
+    snprintf(key, sizeof key, "batch|%d|%d|%d|%d|%d|%d|%p|%p|%p|%p|%p|%p|%p|%p|%p|%p", prec, chunk, (int)reliable,
              sh.site_threads, sh.vec_threads, sh.units, (const void*)t.sys, (const void*)t.ops,
              (const void*)t.hdr, (const void*)t.act, (const void*)t.msite, (const void*)t.mvec,
-             (const void*)t.mupd);
+             (const void*)t.mupd, (const void*)t.vsite, (const void*)t.vvec, (const void*)t.vupd);
     GraphEntry& ge = c->graphs[key];
     if (ge.exec && ge.gen == c->gen) {
         *out = &ge;
@@ -2230,7 +2244,13 @@ extern "C" int msc_solve_batched(msc_ctx* c, int nprob, const msc_problem* probs
     }
     // ---- tables and autotuned launch shape -------------------------------------
     BatchHost bh;
-    st = batch_layout(c, std::max(J, nslots), nprob, bh);
+    int64_t cap_site = 0, cap_vec = 0;  // every slot a system of its own (refinement)
+    for (int g = 0; g < nslots; ++g) {
+        const BSys& q = sys[slot_sys[g]];
+        cap_site += (ops[q.op].g.V + kMinSiteThreads - 1) / kMinSiteThreads;
+        cap_vec += (q.npad + kMinVecThreads - 1) / kMinVecThreads;
+    }
+    st = batch_layout(c, std::max(J, nslots), nprob, cap_site, cap_vec, bh);
     if (st) return st;
     st = upload_systems(c, bh, sys, ops);
     if (st) return st;

@@ -224,6 +224,12 @@ struct BVec {            // base pointers of the batch's vectors
     double2* t64;
     const double2* b64;
 };
+struct alignas(16) VBlock {  // a virtual block
+    int j;               // system
+    int lb;              // block within the system
+    int nb;              // blocks of the system
+    int op;              // its operator
+};
 struct BTab {             // device tables of a batched stage
     const BSys* sys;     // [systems]
     const BOp* ops;      // [operators]
@@ -232,7 +238,12 @@ struct BTab {             // device tables of a batched stage
     const int* msite;    // [active + 1] prefix sums of blocks: operator passes
     const int* mvec;     // [active + 1] one unit per thread (init, fold)
     const int* mupd;     // [active + 1] `units` units per thread (update)
+    const VBlock* vsite; // the virtual blocks of the three maps
+    const VBlock* vvec;
+    const VBlock* vupd;
 };
+// Fills the three tables (at most `blocks` entries in all) from the maps.
+cudaError_t launch_b_expand(const BTab& t, VBlock* vsite, VBlock* vvec, VBlock* vupd, int blocks, cudaStream_t st);
 cudaError_t launch_b_stag(int prec, int kind, int out_f32, const Engine& e, const PassDesc* descs,
                           const BTab& t, int threads, cudaStream_t st);
 cudaError_t launch_b_init(int prec, const Engine& e, const BVec& v, const BTab& t, int threads,
