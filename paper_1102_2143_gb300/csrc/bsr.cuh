@@ -38,6 +38,30 @@ __device__ __forceinline__ void bsr_row(const OpDev& A, const T2<T>* __restrict_
     }
 }
 
+// y = A src for one row of a matrix of real 1 x 1 blocks in FP64 (valsr,
+// [slot][lane]): half the FMAs and half the value bytes. An Inf or NaN among
+// the row's entries would meet the zero imaginary parts, so such a row takes
+// the complex form.
+__device__ __forceinline__ void bsr_row_real(const OpDev& A, const double2* __restrict__ vals,
+                                             const double2* __restrict__ src, int row, double2 (&y)[1]) {
+    const int slice = row >> 5, lane = row & 31;
+    const int len = __ldg(&A.slice_len[slice]);
+    const int64_t st = __ldg(&A.slice_start[slice]);
+    const int32_t* __restrict__ cp = A.cols + st * 32 + lane;
+    const double* __restrict__ vp = A.valsr + st * 32 + lane;
+    unsigned e = 0;
+    y[0] = {0.0, 0.0};
+#pragma unroll 5
+    for (int k = 0; k < len; ++k) {
+        const double2 x = __ldg(src + __ldg(cp + k * 32));
+        const double v = __ldg(vp + k * 32);
+        fx_bound(e, x);
+        y[0].x = fma(v, x.x, y[0].x);
+        y[0].y = fma(v, x.y, y[0].y);
+    }
+    if (e >= 0x7ff00000u) bsr_row<double, 1>(A, vals, src, row, y);
+}
+
 // ---------------------------------------------------------------------------
 // FP64 rows by fixed-point sums (fixed.cuh), bd = 2 and 3. A block is stored as
 // the 28-bit limbs of its entries in units of 2^-56 of the power of two above

@@ -784,7 +784,7 @@ int msc_destroy(msc_ctx* c) {
 
 static void free_op_dev(OpDev& d) {
     // links64 holds the staggered operator's one allocation
-    void* ps[] = {d.links64, d.slice_len, d.slice_start, d.cols, d.vals64, d.valsfx, d.blkfx, d.vals32};
+    void* ps[] = {d.links64, d.slice_len, d.slice_start, d.cols, d.vals64, d.valsr, d.valsfx, d.blkfx, d.vals32};
     for (void* p : ps)
         if (p) cudaFree(p);
     memset(&d, 0, sizeof d);
@@ -989,7 +989,13 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
     if (e != cudaSuccess) return fail(cuda_status(e));
     if (bad & 1) return fail(MSC_ERR_ARG);
-    if (bad) {  // some block does not fit the limbs: the whole matrix in FP64
+    if (bd == 1 && !(bad & 4)) {
+        e = cudaMalloc((void**)&d.valsr, 8 * 32 * std::max<int64_t>(acc, 1));
+        if (e == cudaSuccess) e = bsr_pack_real(d, c->work);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
+        if (e != cudaSuccess) return fail(cuda_status(e));
+    }
+    if (bad & 2) {  // some block does not fit the limbs: the whole matrix in FP64
         cudaFree(d.valsfx);
         cudaFree(d.blkfx);
         d.valsfx = nullptr;

@@ -62,6 +62,7 @@ struct OpDev {
     int64_t* slice_start;
     int32_t* cols;      // [slot][32]
     double2* vals64;    // [slot][bd*bd][32]; null where valsfx is used
+    double* valsr;      // bd = 1, all entries real: their real parts [slot][32]; else null
     int4* valsfx;       // bd > 1: fixed-point limbs [slot][bd*bd][32] (see bsr.cuh); else null
     uint16_t* blkfx;    // and the blocks' exponents [slot][32]
     float2* vals32;
@@ -188,10 +189,12 @@ cudaError_t stag_export_bsr(const OpDev& op, int64_t* row_ptr, int32_t* col, dou
 // patterns; d_out zeroed by the caller).
 cudaError_t bsr_check_hermitian(const int64_t* d_row_ptr, const int32_t* d_col, const double2* d_vals,
                                 int64_t nbr, int bd, unsigned long long* d_out, cudaStream_t st);
+// The real parts of a matrix of 1 x 1 blocks (valsr from vals64).
+cudaError_t bsr_pack_real(OpDev& op, cudaStream_t st);
 // Packs columns, vals32 and whichever of vals64 and valsfx is allocated; sets
-// bit 0 of *d_bad on a column out of range and bit 1 on a block that limbs
+// bit 0 of *d_bad on a column out of range, bit 1 on a block that limbs
 // cannot hold (entries that are not finite, or near the ends of the exponent
-// range).
+// range) and bit 2 on an entry that is not real.
 cudaError_t bsr_pack(OpDev& op, const int64_t* d_row_ptr, const int32_t* d_col,
                      const double2* d_vals, int* d_bad, cudaStream_t st);
 

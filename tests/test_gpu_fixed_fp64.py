@@ -239,3 +239,26 @@ def test_apply_in_place_overlapping_and_unaligned(ctx, bsr):
         y = x.clone()
         msc.msc_op_dslash(ctx, op, y, y)
         assert torch.equal(y, d)
+
+
+def test_real_1x1_rows_equal_complex_rows(ctx):
+    """A matrix of real 1 x 1 entries (ragged, with padding) against the oracle
+    in FP64 (1e-13: rounding order only), with an Inf among the entries of x as
+    the complex form has it, and one imaginary entry, which leaves the path."""
+    n = 77
+    rp, ci, va, _ = inputs.random_hpd_bsr(n, 1, 5, 0.5, 97)
+    va = np.ascontiguousarray(va.real.astype(complex))
+    v = inputs.gaussian_source(n, 98)
+    for imag in (0.0, 0.25):
+        w = va.copy()
+        w[3, 0, 0] += 1j * imag
+        op = msc.msc_op_bsr(ctx, n, 1, rp, ci, w)
+        for x in (v, np.where(np.arange(n) == 40, np.inf + 1j, v)):
+            out = np.empty_like(v)
+            msc.msc_op_apply(ctx, op, 0.3, x, out, msc.MSC_FP64)
+            want = oracle.bsr_apply(rp, ci, w, x, 0.3)
+            ok = np.isfinite(want)
+            # rows shorter than their slice's longest are padded with zeros on column 0
+            assert np.array_equal(ok, np.isfinite(out))
+            assert np.linalg.norm(out[ok] - want[ok]) <= 1e-13 * np.linalg.norm(want[ok])
+        msc.msc_op_destroy(op)
