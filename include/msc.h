@@ -49,9 +49,10 @@ extern "C" {
 #define MSC_ERR_NOT_HPD       4  /* p^dagger A p <= 0 met: A is not positive definite */
 #define MSC_ERR_NONFINITE     5  /* NaN or Inf met in the source or the iteration */
 #define MSC_ERR_NOT_CONVERGED 6  /* iteration cap reached; x is written, see info */
-#define MSC_ERR_TIMEOUT       7  /* a kernel's bounded wait on its own asynchronous
-                                    copies ran out (the solve's results are void;
-                                    the context stays usable) */
+#define MSC_ERR_TIMEOUT       7  /* a kernel's bounded wait (on its own asynchronous
+                                    copies, or on the other blocks of a
+                                    cooperative launch) ran out (the solve's
+                                    results are void; the context stays usable) */
 #define MSC_ERR_UNSUPPORTED   8  /* valid request the library does not handle */
 #define MSC_ERR_BREAKDOWN     9  /* msc_solve_nonherm: a BiCGStab denominator vanished */
 
@@ -215,7 +216,8 @@ typedef struct {
                   fused |r|^2; staggered: second D pass with r -= alpha Ap
                   and |r|^2 fused),
        update_ms  the fused multi-shift update kernel;
-       prof_samples the number of samples (0: not measured);
+       prof_samples the number of samples (0: not measured, as on small
+                  staggered systems, whose iterations share one kernel);
        prof_active  the mean, over the samples, of the number of non-base
                   shifts (summed over right-hand sides) still iterating at
                   the sampled iteration: the sampled update kernel moved
