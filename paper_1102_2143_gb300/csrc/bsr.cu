@@ -21,6 +21,7 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
                            uint16_t* __restrict__ efx, int* bad) {
     const int e2 = bd * bd;
     const int64_t nrow_pad = ((nbr + 31) / 32) * 32;
+    int found = 0;
     for (int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; row < nrow_pad;
          row += (int64_t)gridDim.x * blockDim.x) {
         const int64_t slice = row >> 5;
@@ -34,7 +35,7 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
             int c = 0;
             if (k < rl) {
                 c = col[b0 + k];
-                if (c < 0 || (int64_t)c >= nbr) { atomicOr(bad, 1); c = 0; }
+                if (c < 0 || (int64_t)c >= nbr) { found |= 1; c = 0; }
             }
             pcol[slot * 32 + lane] = c;
             int ex = 0;
@@ -47,13 +48,13 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
                     zero = zero && v.x == 0.0 && v.y == 0.0;
                 }
                 ex = zero ? 0 : (int)(e >> 20);
-                if (!zero && (ex < 200 || ex > 1900)) { atomicOr(bad, 2); ex = 1023; }
+                if (!zero && (ex < 200 || ex > 1900)) { found |= 2; ex = 1023; }
                 efx[slot * 32 + lane] = (uint16_t)ex;
             }
             for (int q = 0; q < e2; ++q) {
                 double2 v = {0.0, 0.0};
                 if (k < rl) v = vals[(b0 + k) * e2 + q];
-                if (bd == 1 && !(v.y == 0.0)) atomicOr(bad, 4);
+                if (bd == 1 && !(v.y == 0.0)) found |= 4;
                 if (v64) v64[(slot * e2 + q) * 32 + lane] = v;
                 v32[(slot * e2 + q) * 32 + lane] = make_float2((float)v.x, (float)v.y);
                 if (vfx) {
@@ -66,6 +67,7 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
             }
         }
     }
+    if (found & ~*(volatile int*)bad) atomicOr(bad, found);
 }
 
 __global__ void k_pack_real(const double2* __restrict__ in, double* __restrict__ out, int64_t n) {

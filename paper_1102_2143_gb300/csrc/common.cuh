@@ -548,6 +548,13 @@ __device__ __forceinline__ SysBlock sys_block(int nsys, const int* act) {
             return s;
         }
     }
+    if (nsys == 1) {  // the list can hold no other (its two loads would come before every other)
+        s.j = 0;
+        s.bx = blockIdx.x;
+        s.gx = gridDim.x;
+        s.ok = true;
+        return s;
+    }
     const int na = act ? __ldg(act) : nsys;
     s.ok = na > 0;
     if (!s.ok) { s.j = s.bx = s.gx = 0; return s; }
