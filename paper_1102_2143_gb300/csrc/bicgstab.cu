@@ -39,9 +39,7 @@ __device__ bool reduce3_last(const Engine& e, int row0, double a, double b, doub
         const double t = warp_total<double>((int)blockDim.x, [&](int i) { return sv[q][i]; });
         if (threadIdx.x == 0) part[(size_t)q * kMaxBlocks + blockIdx.x] = t;
     }
-    int last = 0;
-    if (threadIdx.x == 0) last = arrive(&e.counter[row0]) == gridDim.x - 1;
-    if (!__shfl_sync(0xffffffffu, last, 0)) return false;
+    if (!warp_arrive_last(&e.counter[row0], (int)gridDim.x)) return false;
 #pragma unroll
     for (int q = 0; q < 3; ++q) tot[q] = sum_partials(part + (size_t)q * kMaxBlocks, (int)gridDim.x);
     if (threadIdx.x == 0) e.counter[row0] = 0u;
@@ -162,7 +160,7 @@ __global__ void __launch_bounds__(FX ? 128 : kThreads, FX ? 4 : 3) k_bcg_op(OpDe
             if (!cfinite(zn) || !cfinite(Tn) || czero(q->a_s)) bad = 1;
         }
     }
-    bad = __any_sync(0xffffffffu, bad);
+    bad = warp_any(bad);
     if (threadIdx.x == 0) {
         if (!ok) sys->status = ST_ERR_NONFINITE;
         else if (!(tt > 0.0) || czero(omega) || bad) sys->status = ST_ERR_BREAKDOWN;
@@ -221,7 +219,7 @@ __global__ void __launch_bounds__(kThreads) k_bcg_r(Engine e, BcgSys* sys, BcgSl
         q->T = q->T_new;
         if (q->conv_iter < 0) all = 0;
     }
-    all = __all_sync(0xffffffffu, all);
+    all = warp_all(all);
     if (threadIdx.x == 0) {
         sys->rnorm2 = R;
         sys->beta = beta;

@@ -297,6 +297,32 @@ __device__ __forceinline__ unsigned arrive(unsigned* counter) {
     return t;
 }
 
+// Whether the condition holds in every / any lane, with every lane's earlier
+// memory accesses done before any lane's later ones (a vote alone orders none:
+// lane 0 goes on to overwrite scalars that the others have read).
+__device__ __forceinline__ int warp_all(int v) {
+    const int all = __all_sync(0xffffffffu, v);
+    __syncwarp();
+    return all;
+}
+__device__ __forceinline__ int warp_any(int v) {
+    const int any = __any_sync(0xffffffffu, v);
+    __syncwarp();
+    return any;
+}
+
+// Counts the calling block's arrival (warp 0, all its lanes); true in every
+// lane in the last of `nblocks` blocks. A shuffle hands the count on but orders
+// no memory, so the barrier after it is what lets the other lanes read what the
+// other blocks published before they arrived.
+__device__ __forceinline__ bool warp_arrive_last(unsigned* counter, int nblocks) {
+    int last = 0;
+    if ((threadIdx.x & 31) == 0) last = arrive(counter) == (unsigned)nblocks - 1;
+    last = __shfl_sync(0xffffffffu, last, 0);
+    __syncwarp();
+    return last != 0;
+}
+
 // Publishes this block's sum of v to row `row`; returns true in every lane of
 // warp 0 of the last of the `nblocks` blocks that reduce into that row to
 // arrive (`bidx` = this block's index among them), with the fixed-order total.
@@ -306,12 +332,8 @@ __device__ __forceinline__ bool reduce_last_n(const Engine& e, int row, T v, dou
     const double s = block_sum(v, sv);
     if (threadIdx.x >= 32) return false;
     double* part = e.partial + (size_t)row * kMaxBlocks;
-    int last = 0;
-    if (threadIdx.x == 0) {
-        part[bidx] = s;
-        last = arrive(&e.counter[row]) == (unsigned)nblocks - 1;
-    }
-    if (!__shfl_sync(0xffffffffu, last, 0)) return false;
+    if (threadIdx.x == 0) part[bidx] = s;
+    if (!warp_arrive_last(&e.counter[row], nblocks)) return false;
     total = sum_partials(part, nblocks);
     if (threadIdx.x == 0) e.counter[row] = 0u;
     return true;
@@ -414,7 +436,7 @@ __device__ __forceinline__ void fin_R(const Engine& e, int j, double Rn) {
         q->zeta = zn;
         if (q->conv_iter < 0) all = 0;
     }
-    all = __all_sync(0xffffffffu, all);
+    all = warp_all(all);
     if (lane == 0) {
         s->alpha_prev = alpha;
         s->beta_prev = beta;
