@@ -119,10 +119,11 @@ __device__ __forceinline__ size_t vix(int x, int a, int V) {
     return (PL && sizeof(T) == 4) ? (size_t)a * V + x : (size_t)x * NC + a;
 }
 
-// y = D src at site x
+// y = D src at site x. src may have been written by other blocks of the same
+// kernel: it is neither restrict nor read through the read-only path.
 template <class T, int NC, int RECON, bool PL = false>
-__device__ __forceinline__ void dslash_site(const void* links, const T2<T>* __restrict__ src, int x,
-                                            const StagGeom& g, T2<T> (&y)[NC]) {
+__device__ __forceinline__ void dslash_site_fresh(const void* links, const T2<T>* src, int x, const StagGeom& g,
+                                                  T2<T> (&y)[NC]) {
     const SiteNbrs nb = neighbours(x, g);
 #pragma unroll
     for (int a = 0; a < NC; ++a) y[a] = {T(0), T(0)};
@@ -151,6 +152,13 @@ __device__ __forceinline__ void dslash_site(const void* links, const T2<T>* __re
     }
 }
 
+// The same of a vector that nothing writes while the kernel runs.
+template <class T, int NC, int RECON, bool PL = false>
+__device__ __forceinline__ void dslash_site(const void* links, const T2<T>* __restrict__ src, int x, const StagGeom& g,
+                                            T2<T> (&y)[NC]) {
+    dslash_site_fresh<T, NC, RECON, PL>(links, src, x, g, y);
+}
+
 // y = D src at site x in FP64 on the FP64 pipe, for the sites whose entries
 // leave the range of the fixed-point sums (rare: out of line).
 template <int NC> struct SiteVec {
@@ -159,7 +167,7 @@ template <int NC> struct SiteVec {
 template <int NC>
 __device__ __noinline__ SiteVec<NC> dslash_site_f64(const void* links64, const double2* src, int x, const StagGeom& g) {
     SiteVec<NC> r;
-    dslash_site<double, NC, 0>(links64, src, x, g, r.y);
+    dslash_site_fresh<double, NC, 0>(links64, src, x, g, r.y);
     return r;
 }
 
@@ -183,8 +191,7 @@ __host__ __device__ __forceinline__ size_t fx_link(int mu, int x, int V) {
 // FRESH: src may have been written by other blocks of the same kernel, so its
 // loads do not take the read-only path.
 template <int NC, bool FRESH>
-__device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* links64, const double2* __restrict__ src,
-                                               int x, const StagGeom& g, double2 (&y)[NC]) {
+__device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* links64, const double2* src, int x, const StagGeom& g, double2 (&y)[NC]) {
     if (!lfx) {  // links that are not unitary (batches mix operators)
         const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
 #pragma unroll
@@ -274,9 +281,8 @@ using SiteAcc = typename std::conditional<(sizeof(T) == 4 && KIND != PASS_C), fl
 // The epilogue KIND of a D pass at colour a of vector site x, y = (D src)_a
 // there; adds to the site's share of the reduction (nothing when d.row < 0).
 template <class T, int NC, int KIND, class TO, bool PL>
-__device__ __forceinline__ void stag_colour(const PassDesc& d, int x, int a, int V, T2<T> y, T alpha,
-                                            SiteAcc<T, KIND>& loc) {
-    const T2<T>* __restrict__ aux = (const T2<T>*)d.aux;
+__device__ __forceinline__ void stag_colour_of(const PassDesc& d, const T2<T>* aux, int x, int a, int V, T2<T> y,
+                                               T alpha, SiteAcc<T, KIND>& loc) {
     const T dd = (T)d.d;
     const size_t i = vix<T, PL, NC>(x, a, V);
     if (KIND == PASS_A) {
@@ -312,21 +318,33 @@ __device__ __forceinline__ void stag_colour(const PassDesc& d, int x, int a, int
     }
 }
 
+// (FRESH: d.aux, like the source, may be another block's of the same kernel.)
+template <class T, int NC, int KIND, class TO, bool PL, bool FRESH>
+__device__ __forceinline__ void stag_colour(const PassDesc& d, int x, int a, int V, T2<T> y, T alpha,
+                                            SiteAcc<T, KIND>& loc) {
+    if constexpr (FRESH) {
+        stag_colour_of<T, NC, KIND, TO, PL>(d, (const T2<T>*)d.aux, x, a, V, y, alpha, loc);
+    } else {
+        const T2<T>* __restrict__ aux = (const T2<T>*)d.aux;
+        stag_colour_of<T, NC, KIND, TO, PL>(d, aux, x, a, V, y, alpha, loc);
+    }
+}
+
 // RECON = kLinksFx (FP64 only): `links` holds fixed-point limbs and links64
-// the FP64 links.
+// the FP64 links. FRESH: see dslash_site_fresh.
 constexpr int kLinksFx = 2;
 template <class T, int NC, int RECON, int KIND, class TO, bool PL = false, bool FRESH = false>
 __device__ __forceinline__ SiteAcc<T, KIND> stag_site(const PassDesc& d, const StagGeom& g, const void* links,
                                             T alpha, int x, const void* links64 = nullptr) {
-    const T2<T>* __restrict__ src = (const T2<T>*)d.src;
     const int V = vlen(g);
     T2<T> y[NC];
-    if constexpr (RECON == kLinksFx) dslash_site_fx<NC, FRESH>(links, links64, src, x, g, y);
-    else dslash_site<T, NC, RECON, PL>(links, src, x, g, y);
+    if constexpr (RECON == kLinksFx) dslash_site_fx<NC, FRESH>(links, links64, (const T2<T>*)d.src, x, g, y);
+    else if constexpr (FRESH) dslash_site_fresh<T, NC, RECON, PL>(links, (const T2<T>*)d.src, x, g, y);
+    else dslash_site<T, NC, RECON, PL>(links, (const T2<T>*)d.src, x, g, y);
     x = vsite(x, g);  // the site's index in the vectors
     SiteAcc<T, KIND> loc = 0;
 #pragma unroll
-    for (int a = 0; a < NC; ++a) stag_colour<T, NC, KIND, TO, PL>(d, x, a, V, y[a], alpha, loc);
+    for (int a = 0; a < NC; ++a) stag_colour<T, NC, KIND, TO, PL, FRESH>(d, x, a, V, y[a], alpha, loc);
     return loc;
 }
 
@@ -338,7 +356,7 @@ __device__ __forceinline__ SiteAcc<T, KIND> stag_site(const PassDesc& d, const S
 template <int NC, int KIND, class TO, bool FRESH>
 __device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeom& g, const void* lfx,
                                                 const void* links64, double alpha, int x, bool on) {
-    const double2* __restrict__ src = (const double2*)d.src;
+    const double2* src = (const double2*)d.src;
     const int mu = threadIdx.x & 3;
     const int q0 = gdiv(x, g, 0), q1 = gdiv(q0, g, 1), q2 = gdiv(q1, g, 2);
     const int c0 = x - q0 * g.L[0], c1 = q0 - q1 * g.L[1], c2 = q1 - q2 * g.L[2];
@@ -412,7 +430,7 @@ __device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeo
             if (a == mu) y = r.y[a];
     }
     double loc = 0.0;
-    stag_colour<double, NC, KIND, TO, true>(d, vsite(x, g), mu, vlen(g), y, alpha, loc);
+    stag_colour<double, NC, KIND, TO, true, FRESH>(d, vsite(x, g), mu, vlen(g), y, alpha, loc);
     return loc;
 }
 

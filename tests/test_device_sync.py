@@ -25,3 +25,21 @@ def test_votes_and_broadcast_decisions_are_followed_by_a_warp_barrier():
             end = text.index(";", m.end())
             assert re.match(r"\s*__syncwarp\(\);", text[end + 1:]), (name, text[m.start():end + 1])
     assert seen >= 3
+
+
+def test_vectors_that_other_blocks_write_are_not_read_as_constant():
+    """The cooperative iterations (FRESH) gather vectors that other blocks of
+    the same kernel wrote: the functions on that path hold them in plain
+    pointers, and the read-only path is for links or for FRESH = false."""
+    text = dict(sources())["stencil.cuh"]
+    for fn in ("dslash_site_fresh", "dslash_site_f64", "dslash_site_fx", "stag_colour_of", "stag_site", "stag_site_fx4"):
+        at = re.search(r"__device__ \w+ (?:SiteAcc<T, KIND>|SiteVec<NC>|\w+) " + fn + r"\(", text).start()
+        end = text.find("\ntemplate", at)
+        body = text[at:end if end > 0 else None]
+        assert not re.search(r"__restrict__ (?:src|aux|v[fb])\b", body), fn
+        for m in re.finditer(r"__ldg\((\w+)", body):
+            line = body[body.rfind("\n", 0, m.start()):m.start()]
+            assert m.group(1) == "U" or "FRESH ?" in line, (fn, line)
+        if fn != "dslash_site_fresh":
+            plain = re.search(r"\bdslash_site<", body)
+            assert not plain or "if constexpr (FRESH) dslash_site_fresh" in body, fn
