@@ -86,9 +86,10 @@ struct msc_ctx {
     Buf errf;         // device error word (bit 0: a bounded wait in a kernel ran out), then
                       // scratch words of the operators' set-up (offsets kSetupWord, kSetupMax)
     unsigned* h_err = nullptr;  // pinned copy of it
-    uint64_t wait_ns = 2000000000ull;  // limit of a kernel's wait on its own copies
+    uint64_t wait_ns = 2000000000ull;  // limit of a kernel's wait on its own copies or grid barrier
     int use_tile = 0;  // one-system FP32 stencil passes stage their links (when the lattice tiles)
     int test_no_copy = 0;  // tests only: the staged passes issue no copies, so their waits run out
+    int test_absent = 0;   // tests only: grid barriers wait for an arrival that never comes
     int use_cond = 1; // build reliable updates as conditional graph nodes
     int* h_flags = nullptr;  // pinned copy of the conditional flags of a chunk
     int* h_act = nullptr;
@@ -503,6 +504,7 @@ static int run_stage_persist(msc_ctx* c, const msc_op* op, int prec, int nsys, i
     a.links64 = A.links64;
     a.bar = (unsigned*)c->gbar.p;
     a.wait_ns = c->wait_ns;
+    a.absent = (unsigned)c->test_absent;
     a.nsys = nsys;
     a.nslots = nslots;
     a.iters = reliable ? 50 : 100;
@@ -723,14 +725,17 @@ int msc_create(msc_ctx** out, int device, void* stream) {
     // MSC_STAG_TILE=1: one-system FP32 stencil passes stage their links in
     // shared memory by bulk asynchronous copies (lattices that tile; off by
     // default, the direct passes are faster). MSC_WAIT_NS: the limit of a
-    // kernel's wait on its own asynchronous copies. MSC_TEST_NO_COPY=1 (tests
-    // of the timeout path only): the staged passes issue no copies.
+    // kernel's wait on its own asynchronous copies or, in a cooperative launch,
+    // on the other blocks. For tests of the timeout paths only:
+    // MSC_TEST_NO_COPY=1, the staged passes issue no copies; MSC_TEST_ABSENT=1,
+    // the grid barriers wait for one arrival more than there are.
     if (const char* ev = getenv("MSC_STAG_TILE")) c->use_tile = atoi(ev) != 0;
     if (const char* ev = getenv("MSC_WAIT_NS")) {
         const long long w = atoll(ev);
         if (w > 0) c->wait_ns = (uint64_t)w;
     }
     if (const char* ev = getenv("MSC_TEST_NO_COPY")) c->test_no_copy = atoi(ev) != 0;
+    if (const char* ev = getenv("MSC_TEST_ABSENT")) c->test_absent = atoi(ev) != 0;
     cudaError_t e = cudaStreamCreateWithFlags(&c->work, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_sync, cudaEventDisableTiming);
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&c->prof[i]);

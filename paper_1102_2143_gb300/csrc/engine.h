@@ -131,7 +131,8 @@ struct VecSet {
 // (persist.cu): all nsys systems (whose shifts lie in the first nslots slots)
 // run until every one has stopped, one of them is due a reliable update, or
 // `iters` iterations are done. k1, k2: the pass descriptors (device). bar: a
-// barrier word, zeroed before each launch. persist_applies() says whether a
+// barrier word, zeroed before each launch. absent: 0, or (tests) the number of
+// arrivals that every barrier waits for in vain. persist_applies() says whether a
 // stage takes this path.
 struct PersistArgs {
     Engine e;
@@ -143,6 +144,7 @@ struct PersistArgs {
     const void* links64;
     unsigned* bar;
     uint64_t wait_ns;
+    unsigned absent;
     int nsys, nslots, iters;
 };
 bool persist_applies(const OpDev& op, int prec, int nsys, int nslots);

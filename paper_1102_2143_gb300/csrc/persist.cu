@@ -23,7 +23,8 @@
 // 5.4 ms. FP64 (fixed-point passes): 4^4 16 us, 8^4 17 us.
 //
 // Barrier waits are bounded by the global timer (wait_ns): a wait that runs
-// out sets the context's error word and the block returns.
+// out sets the context's error word and the block returns; launches queued
+// behind it find the word set and return at once.
 #include <algorithm>
 
 #include "async.cuh"
@@ -149,11 +150,14 @@ __global__ void __launch_bounds__(kThreads, BPS) k_persist(PersistArgs a) {
     PassDesc* k2 = k1 + nsys;
     SysCoefs<T>* cy = (SysCoefs<T>*)(k2 + nsys);
     ShiftCoefs<T>* cs = (ShiftCoefs<T>*)(((uintptr_t)(cy + nsys) + 15) / 16 * 16);
+    __shared__ unsigned s_err;
+    if (threadIdx.x == 0) s_err = a.e.err ? ld_acquire(a.e.err) : 0u;
     copy_words(ss, a.e.sys, nsys);
     copy_words(sl, a.e.slot, a.nslots);
     copy_words(k1, a.k1, nsys);
     copy_words(k2, a.k2, nsys);
     __syncthreads();
+    if (s_err) return;  // an earlier launch's wait ran out: its results are void
     Engine e = a.e;
     e.sys = ss;
     e.slot = sl;
@@ -165,7 +169,7 @@ __global__ void __launch_bounds__(kThreads, BPS) k_persist(PersistArgs a) {
     const int64_t upv = a.v.npad / U16<T>::cpu;
     const int vchunks = (int)((upv + kThreads - 1) / kThreads);
     const int nvtask = nsys * vchunks;
-    GridBar bar{a.bar, 0u, a.wait_ns, a.e.err};
+    GridBar bar{a.bar, a.absent, a.wait_ns, a.e.err};
     bool fine = true;
     for (int it = 0; it < a.iters; ++it) {
         bool go = false, ru = false;
