@@ -717,6 +717,10 @@ __global__ void k_packfx(const double2* __restrict__ in, int4* __restrict__ out,
     }
 }
 
+// The larger of two deviations; one that is not a number counts as 1e300 (fmax
+// would drop it, and a link with a NaN would pass for a unitary one).
+__device__ __forceinline__ double worse(double m, double d) { return d <= m ? m : d == d ? d : 1e300; }
+
 // max over links of max(|U U^dag - 1|_max, |det U - 1|)
 __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlinks,
                             unsigned long long* maxdev) {
@@ -729,7 +733,7 @@ __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlin
                 double2 s = {0.0, 0.0};
                 for (int c = 0; c < nc; ++c) s = cadd(s, cmul(u[a * nc + c], cconj(u[b * nc + c])));
                 if (a == b) s.x -= 1.0;
-                m = fmax(m, fmax(fabs(s.x), fabs(s.y)));
+                m = worse(worse(m, fabs(s.x)), fabs(s.y));
             }
         double2 det;
         if (nc == 2) {
@@ -740,8 +744,7 @@ __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlin
             det = cadd(det, cmul(u[2], csub(cmul(u[3], u[7]), cmul(u[4], u[6]))));
         }
         det.x -= 1.0;
-        m = fmax(m, fmax(fabs(det.x), fabs(det.y)));
-        if (!(m == m)) m = 1e300;
+        m = worse(worse(m, fabs(det.x)), fabs(det.y));
     }
     // non-negative doubles order like their bit patterns; one atomic per warp
     // (one per link on one address made it 200 us at 16^4, and the set-up of a
