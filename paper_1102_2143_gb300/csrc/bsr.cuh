@@ -147,10 +147,13 @@ __device__ __forceinline__ void bsr_row_fx(const OpDev& A, const double2* __rest
 #pragma unroll
                 for (int b = 0; b < BD; ++b) fx_bound(e, x[j][b]);
                 finite = finite && e < 0x7ff00000u;
+                // a block that meets zeros only is like a zero block: taken at the
+                // row's own exponent, far above any entry's, so that fx_split gives 0
+                if (e == 0) eb[j] = 0;
                 if (e < (64u << 20))  // zeros, or next to the subnormals
 #pragma unroll
                     for (int b = 0; b < BD; ++b) finite = finite && x[j][b].x == 0.0 && x[j][b].y == 0.0;
-                if (e != 0 && eb[j] != 0) top = max(top, (int)(e >> 20) + eb[j]);
+                if (eb[j] != 0) top = max(top, (int)(e >> 20) + eb[j]);
             }
         FxSum re[BD], im[BD];
 #pragma unroll
