@@ -13,13 +13,47 @@
 
 namespace msc {
 
+// Whether limbs hold a block row (p: its largest parts per place (a, b) of a
+// block, as exponent bounds). A block's limbs are in units of 2^-56 of its
+// largest part and its sums in units of the row's largest products, so entries
+// and sums that are small beside those keep fewer bits than FP64 gives them.
+// In every component's row and column some entry has to be within 2^-4 of the
+// row's largest (what the limbs lose is then 2^-52 of an entry of the same row
+// and of the same column, as in an FP64 rounding), and every pair of
+// components has to be coupled by some entry within 2^-24 (no component's sum
+// is far below the unit by itself). The exported staggered operator meets both
+// at every row (its diagonal block is m^2 + 2 and its hops couple all colours);
+// matrices in mixed units or of independent components do not.
+constexpr unsigned kRowSpan = 4u << 20, kPairSpan = 24u << 20;
+template <int BD>
+__device__ __forceinline__ bool bsr_even_row(const unsigned (&p)[BD * BD]) {
+    unsigned r[BD], c[BD], big = 0, least = ~0u;
+#pragma unroll
+    for (int a = 0; a < BD; ++a) r[a] = c[a] = 0;
+#pragma unroll
+    for (int a = 0; a < BD; ++a)
+#pragma unroll
+        for (int b = 0; b < BD; ++b) {
+            r[a] = max(r[a], p[a * BD + b]);
+            c[b] = max(c[b], p[a * BD + b]);
+            least = min(least, p[a * BD + b]);
+        }
+#pragma unroll
+    for (int a = 0; a < BD; ++a) big = max(big, r[a]);
+    bool even = least + kPairSpan >= big;
+#pragma unroll
+    for (int a = 0; a < BD; ++a) even = even && r[a] + kRowSpan >= big && c[a] + kRowSpan >= big;
+    return even;
+}
+
+template <int BD>
 __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                           const double2* __restrict__ vals, int64_t nbr, int bd,
+                           const double2* __restrict__ vals, int64_t nbr,
                            const int32_t* __restrict__ slice_len,
                            const int64_t* __restrict__ slice_start, int32_t* __restrict__ pcol,
                            double2* __restrict__ v64, float2* __restrict__ v32, int4* __restrict__ vfx,
                            uint16_t* __restrict__ efx, int* bad) {
-    const int e2 = bd * bd;
+    constexpr int bd = BD, e2 = bd * bd;
     const int64_t nrow_pad = ((nbr + 31) / 32) * 32;
     int found = 0;
     for (int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; row < nrow_pad;
@@ -30,6 +64,9 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
         const int64_t st = slice_start[slice];
         const int64_t b0 = row < nbr ? row_ptr[row] : 0;
         const int64_t rl = row < nbr ? row_ptr[row + 1] - b0 : 0;
+        unsigned part[e2];
+#pragma unroll
+        for (int q = 0; q < e2; ++q) part[q] = 0;
         for (int k = 0; k < len; ++k) {
             const int64_t slot = st + k;
             int c = 0;
@@ -42,8 +79,11 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
             if (vfx) {
                 unsigned e = 0;
                 bool zero = true;
-                for (int q = 0; q < e2 && k < rl; ++q) {
+#pragma unroll
+                for (int q = 0; q < e2; ++q) {
+                    if (k >= rl) continue;
                     const double2 v = vals[(b0 + k) * e2 + q];
+                    fx_bound(part[q], v);
                     fx_bound(e, v);
                     zero = zero && v.x == 0.0 && v.y == 0.0;
                 }
@@ -51,6 +91,7 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
                 if (!zero && (ex < 200 || ex > 1900)) { found |= 2; ex = 1023; }
                 efx[slot * 32 + lane] = (uint16_t)ex;
             }
+#pragma unroll
             for (int q = 0; q < e2; ++q) {
                 double2 v = {0.0, 0.0};
                 if (k < rl) v = vals[(b0 + k) * e2 + q];
@@ -66,6 +107,7 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
                 }
             }
         }
+        if (vfx && !bsr_even_row<BD>(part)) found |= 2;
     }
     if (found & ~*(volatile int*)bad) atomicOr(bad, found);
 }
@@ -141,8 +183,9 @@ cudaError_t bsr_pack(OpDev& op, const int64_t* d_row_ptr, const int32_t* d_col,
     int64_t b = (rows + 255) / 256;
     if (b > 65535) b = 65535;
     if (b < 1) b = 1;
-    k_bsr_pack<<<(int)b, 256, 0, st>>>(d_row_ptr, d_col, d_vals, op.nbr, op.bd, op.slice_len,
-                                        op.slice_start, op.cols, op.vals64, op.vals32, op.valsfx, op.blkfx, d_bad);
+    auto k = op.bd == 1 ? k_bsr_pack<1> : op.bd == 2 ? k_bsr_pack<2> : k_bsr_pack<3>;
+    k<<<(int)b, 256, 0, st>>>(d_row_ptr, d_col, d_vals, op.nbr, op.slice_len, op.slice_start, op.cols, op.vals64,
+                              op.vals32, op.valsfx, op.blkfx, d_bad);
     return cudaGetLastError();
 }
 

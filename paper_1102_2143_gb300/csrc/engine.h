@@ -194,9 +194,10 @@ cudaError_t bsr_check_hermitian(const int64_t* d_row_ptr, const int32_t* d_col, 
 // The real parts of a matrix of 1 x 1 blocks (valsr from vals64).
 cudaError_t bsr_pack_real(OpDev& op, cudaStream_t st);
 // Packs columns, vals32 and whichever of vals64 and valsfx is allocated; sets
-// bit 0 of *d_bad on a column out of range, bit 1 on a block that limbs
-// cannot hold (entries that are not finite, or near the ends of the exponent
-// range) and bit 2 on an entry that is not real.
+// bit 0 of *d_bad on a column out of range, bit 1 on a block row that limbs
+// cannot hold (entries that are not finite, near the ends of the exponent
+// range, or far smaller than others of their block row) and bit 2 on an entry
+// that is not real.
 cudaError_t bsr_pack(OpDev& op, const int64_t* d_row_ptr, const int32_t* d_col,
                      const double2* d_vals, int* d_bad, cudaStream_t st);
 
