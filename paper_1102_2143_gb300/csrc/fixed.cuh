@@ -55,8 +55,10 @@ __device__ __forceinline__ bool fx_in_range(unsigned field) {
 }
 
 // v in units of 2^(e - 1078), e the exponent in `field`, truncated; negated
-// where flip = -1 (flip: 0 or -1). Zeros and entries below the unit give 0
-// (the shift is then at least 56).
+// where flip = -1 (flip: 0 or -1). Entries below the unit give 0 (the shift is
+// then at least 56), and so do zeros, whose implicit bit is not masked, when
+// `field` is kFxFloor at least.
+constexpr unsigned kFxFloor = 64u << 20;
 __device__ __forceinline__ void fx_split(double v, unsigned field, int flip, int& h, int& l) {
     const int hi = __double2hiint(v);
     const unsigned lo = (unsigned)__double2loint(v);

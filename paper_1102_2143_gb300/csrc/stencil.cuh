@@ -184,9 +184,10 @@ __host__ __device__ __forceinline__ size_t fx_link(int mu, int x, int V) {
 // fx_link().
 // The sign of eta_mu and of the backward hop goes into the entries' limbs.
 // The entries of one direction (both hops) are loaded and bounded together;
-// the first direction sets the sums' unit with one bit to spare, and a later
-// one with larger entries shifts the sums (about two of three warps do so
-// once on Gaussian entries). Holding all 8 hops' entries for one exact bound
+// the first direction sets the sums' unit with one bit to spare (and not below
+// kFxFloor, where zeros would not be split into zeros: a direction that holds
+// nothing else), and a later one with larger entries shifts the sums (about two
+// of three warps do so once on Gaussian entries). Holding all 8 hops' entries for one exact bound
 // instead needs 255 registers (32^4, two passes: 506 us).
 // FRESH: src may have been written by other blocks of the same kernel, so its
 // loads do not take the read-only path.
@@ -221,7 +222,7 @@ __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* link
         }
         const unsigned f = fx_field(e);
         if (mu == 0) {
-            field = f + (1u << 20);
+            field = max(f + (1u << 20), kFxFloor);
         } else if (f > field) {
             const unsigned d = (f + (1u << 20) - field) >> 20;
             field = f + (1u << 20);
