@@ -160,14 +160,38 @@ __device__ __forceinline__ void dslash_site(const void* links, const T2<T>* __re
 }
 
 // y = D src at site x in FP64 on the FP64 pipe, for the sites whose entries
-// leave the range of the fixed-point sums (rare: out of line).
+// leave the range of the fixed-point sums (rare: out of line). finite: the
+// links are, so a site whose entries are all zero has y = 0 without the sums: a
+// source on one site or one parity stays on alternating parities under D, and
+// half the lanes of every warp of an FP64 pass then come here.
 template <int NC> struct SiteVec {
     double2 y[NC];
 };
 template <int NC>
-__device__ __noinline__ SiteVec<NC> dslash_site_f64(const void* links64, const double2* src, int x, const StagGeom& g) {
+__device__ __noinline__ SiteVec<NC> dslash_site_f64(const void* links64, const double2* src, int x, const StagGeom& g,
+                                                    bool finite) {
     SiteVec<NC> r;
-    dslash_site_fresh<double, NC, 0>(links64, src, x, g, r.y);
+    unsigned long long bits = finite ? 0 : 1;
+    if (finite) {
+        const SiteNbrs nb = neighbours(x, g);
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) {
+            const double2* vf = src + (size_t)vsite(nb.fwd[mu], g) * NC;
+            const double2* vb = src + (size_t)vsite(nb.bwd[mu], g) * NC;
+#pragma unroll
+            for (int b = 0; b < NC; ++b) {
+                const double2 f = vf[b], w = vb[b];
+                bits |= (unsigned long long)(__double_as_longlong(f.x) | __double_as_longlong(f.y) |
+                                             __double_as_longlong(w.x) | __double_as_longlong(w.y)) << 1;
+            }
+        }
+    }
+    if (bits) {
+        dslash_site_fresh<double, NC, 0>(links64, src, x, g, r.y);
+    } else {
+#pragma unroll
+        for (int a = 0; a < NC; ++a) r.y[a] = {0.0, 0.0};
+    }
     return r;
 }
 
@@ -194,7 +218,7 @@ __host__ __device__ __forceinline__ size_t fx_link(int mu, int x, int V) {
 template <int NC, bool FRESH>
 __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* links64, const double2* src, int x, const StagGeom& g, double2 (&y)[NC]) {
     if (!lfx) {  // links that are not unitary (batches mix operators)
-        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g, false);
 #pragma unroll
         for (int a = 0; a < NC; ++a) y[a] = r.y[a];
         return;
@@ -257,7 +281,7 @@ __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* link
         }
     }
     if (!fx_in_range(field)) {
-        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g, true);
 #pragma unroll
         for (int a = 0; a < NC; ++a) y[a] = r.y[a];
         return;
@@ -368,7 +392,7 @@ __device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeo
     const int xf = c == L - 1 ? x - (L - 1) * stride : x + stride;
     const int xb = c == 0 ? x + (L - 1) * stride : x - stride;
     double2 v[2][NC];
-    unsigned e = 0;
+    unsigned e = 0, lows = 0;
 #pragma unroll
     for (int b = 0; b < NC; ++b) {
         v[0][b] = v[1][b] = {0.0, 0.0};
@@ -380,7 +404,10 @@ __device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeo
         }
         fx_bound(e, v[0][b]);
         fx_bound(e, v[1][b]);
+        lows |= (unsigned)__double2loint(v[0][b].x) | (unsigned)__double2loint(v[0][b].y) |
+                (unsigned)__double2loint(v[1][b].x) | (unsigned)__double2loint(v[1][b].y);
     }
+    e = max(e, min(lows, 1u));  // 0 only where every entry is zero
     e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
     e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
     const unsigned field = fx_field(e);
@@ -424,8 +451,10 @@ __device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeo
     }
     if (!on || mu >= NC) return 0.0;
     double2 y = {fx_double(sr, field, 1), fx_double(si, field, 1)};
-    if (!fx_in_range(field)) {
-        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
+    if (e == 0) {
+        y = {0.0, 0.0};
+    } else if (!fx_in_range(field)) {
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g, false);
 #pragma unroll
         for (int a = 0; a < NC; ++a)
             if (a == mu) y = r.y[a];
