@@ -63,7 +63,7 @@ struct Range {
 }  // namespace
 
 // small results of the set-up kernels, behind the context's error word
-constexpr size_t kSetupWord = 4, kSetupMax = 8;
+constexpr size_t kSetupWord = 4, kSetupDev = 8, kErrBytes = kSetupDev + kLinkDevs * sizeof(double);
 
 struct msc_ctx {
     int device = 0;
@@ -84,7 +84,7 @@ struct msc_ctx {
     Buf pb, px0, ptmp;// polynomial right-hand sides: b_s, x_s0, two scratch vectors per shift
     Buf gbar;         // barrier word of the cooperative iterations
     Buf errf;         // device error word (bit 0: a bounded wait in a kernel ran out), then
-                      // scratch words of the operators' set-up (offsets kSetupWord, kSetupMax)
+                      // scratch words of the operators' set-up (offsets kSetupWord, kSetupDev)
     unsigned* h_err = nullptr;  // pinned copy of it
     uint64_t wait_ns = 2000000000ull;  // limit of a kernel's wait on its own copies or grid barrier
     int use_tile = 0;  // one-system FP32 stencil passes stage their links (when the lattice tiles)
@@ -739,10 +739,10 @@ int msc_create(msc_ctx** out, int device, void* stream) {
     cudaError_t e = cudaStreamCreateWithFlags(&c->work, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_sync, cudaEventDisableTiming);
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&c->prof[i]);
-    if (e == cudaSuccess) e = cudaMalloc(&c->errf.p, 16);
+    if (e == cudaSuccess) e = cudaMalloc(&c->errf.p, kErrBytes);
     if (e == cudaSuccess) {
-        c->errf.bytes = 16;
-        e = cudaMemsetAsync(c->errf.p, 0, 16, c->work);
+        c->errf.bytes = kErrBytes;
+        e = cudaMemsetAsync(c->errf.p, 0, kErrBytes, c->work);
     }
     if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_err, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
@@ -858,7 +858,7 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
     const size_t nlink_bytes = (size_t)4 * V * nc * nc * 16;
     const double2* src = (const double2*)links;
     void* tmp = nullptr;
-    double* dmax = (double*)((char*)c->errf.p + kSetupMax);
+    double* ddev = (double*)((char*)c->errf.p + kSetupDev);
     cudaError_t e = cudaSuccess;
     auto fail = [&](cudaError_t err) {
         if (tmp) cudaFree(tmp);
@@ -872,15 +872,17 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
         if (e != cudaSuccess) return fail(e);
         src = (const double2*)tmp;
     }
-    e = cudaMemsetAsync(dmax, 0, sizeof(double), c->work);
-    if (e == cudaSuccess) e = stag_unitarity(d, src, dmax, c->work);
-    double maxdev = 1.0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&maxdev, dmax, sizeof(double), cudaMemcpyDeviceToHost, c->work);
+    double dev[kLinkDevs];
+    e = cudaMemsetAsync(ddev, 0, sizeof dev, c->work);
+    if (e == cudaSuccess) e = stag_unitarity(d, src, ddev, c->work);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dev, ddev, sizeof dev, cudaMemcpyDeviceToHost, c->work);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
     if (e != cudaSuccess) return fail(e);
-    d.recon = (!(flags & MSC_LINKS_FULL) && maxdev < 1e-9) ? 1 : 0;
+    // limbs need entries of at most 1; rebuilding a row needs determinant 1 too
+    const bool unitary = dev[0] < 1e-9;
+    d.recon = (!(flags & MSC_LINKS_FULL) && unitary && dev[1] < 1e-9) ? 1 : 0;
     const size_t l32 = d.recon ? (size_t)4 * V * (nc == 3 ? 3 : 1) * 16 : (size_t)4 * V * nc * nc * 8;
-    const size_t lfx = maxdev < 1e-9 ? (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16 : 0;
+    const size_t lfx = unitary ? (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16 : 0;
     // one allocation for the three forms (each cudaMalloc and cudaFree costs
     // tens of microseconds of a small operator's set-up): FP64, limbs, FP32
     const size_t at_fx = (nlink_bytes + 255) / 256 * 256, at_32 = at_fx + (lfx + 255) / 256 * 256;
@@ -890,7 +892,7 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
     d.links64 = (double2*)block;
     d.linksfx = lfx ? (int4*)(block + at_fx) : nullptr;
     d.links32 = block + at_32;
-    e = stag_pack_links(d, src, dmax, c->work);
+    e = stag_pack_links(d, src, c->work);
     if (e == cudaSuccess) e = stag_pack_links32(d, src, c->work);
     if (e == cudaSuccess && lfx) e = stag_pack_linksfx(d, src, c->work);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);

@@ -721,10 +721,9 @@ __global__ void k_packfx(const double2* __restrict__ in, int4* __restrict__ out,
 // would drop it, and a link with a NaN would pass for a unitary one).
 __device__ __forceinline__ double worse(double m, double d) { return d <= m ? m : d == d ? d : 1e300; }
 
-// max over links of max(|U U^dag - 1|_max, |det U - 1|)
-__global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlinks,
-                            unsigned long long* maxdev) {
-    double m = 0.0;
+// dev[0]: max over links of |U U^dag - 1|_max, dev[1]: of |det U - 1|
+__global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlinks, unsigned long long* dev) {
+    double m = 0.0, md = 0.0;
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < nlinks;
          l += (int64_t)gridDim.x * blockDim.x) {
         const double2* u = in + l * nc * nc;
@@ -744,14 +743,17 @@ __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlin
             det = cadd(det, cmul(u[2], csub(cmul(u[3], u[7]), cmul(u[4], u[6]))));
         }
         det.x -= 1.0;
-        m = worse(worse(m, fabs(det.x)), fabs(det.y));
+        md = worse(worse(md, fabs(det.x)), fabs(det.y));
     }
     // non-negative doubles order like their bit patterns; one atomic per warp
     // (one per link on one address made it 200 us at 16^4, and the set-up of a
     // 27,000-site SU(2) operator 0.2 ms longer)
-    unsigned long long b = (unsigned long long)__double_as_longlong(m);
-    for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(maxdev, b);
+    unsigned long long b[2] = {(unsigned long long)__double_as_longlong(m),
+                               (unsigned long long)__double_as_longlong(md)};
+    for (int k = 0; k < 2; ++k) {
+        for (int o = 16; o > 0; o >>= 1) b[k] = max(b[k], __shfl_xor_sync(0xffffffffu, b[k], o));
+        if ((threadIdx.x & 31) == 0) atomicMax(dev + k, b[k]);
+    }
 }
 
 // FP32 links: full [4][nc*nc][V] float2, or rows [4][k][V] float4 (recon)
@@ -883,18 +885,15 @@ static int setup_blocks(int64_t work) {
     return (int)b;
 }
 
-cudaError_t stag_pack_links(OpDev& op, const double2* links_aos, double* d_maxdev, cudaStream_t st) {
-    (void)d_maxdev;
+cudaError_t stag_pack_links(OpDev& op, const double2* links_aos, cudaStream_t st) {
     const int64_t total = (int64_t)4 * op.g.V * op.nc * op.nc;
     k_pack64<<<setup_blocks(total), 256, 0, st>>>(links_aos, op.links64, op.nc, op.g.V);
     return cudaGetLastError();
 }
 
-cudaError_t stag_unitarity(const OpDev& op, const double2* links_aos, double* d_maxdev,
-                           cudaStream_t st) {
+cudaError_t stag_unitarity(const OpDev& op, const double2* links_aos, double* d_dev, cudaStream_t st) {
     const int64_t nl = (int64_t)4 * op.g.V;
-    k_unitarity<<<setup_blocks(nl), 256, 0, st>>>(links_aos, op.nc, nl,
-                                                  (unsigned long long*)d_maxdev);
+    k_unitarity<<<setup_blocks(nl), 256, 0, st>>>(links_aos, op.nc, nl, (unsigned long long*)d_dev);
     return cudaGetLastError();
 }
 
