@@ -832,6 +832,21 @@ static int begin(msc_ctx* c) {
     return MSC_OK;
 }
 
+// Whether the device has room for an optional second copy of `bytes` of an
+// operator's data beside the `needed` bytes that it cannot do without. A copy
+// serves speed alone: it may not make an operator or a solve fail that fits
+// without it, so eight times its size has to stay free for the solves. (The
+// query is left out for copies that no card is short of.)
+static bool room_for_copy(size_t bytes, size_t needed) {
+    if (bytes <= (size_t)64 << 20) return true;
+    size_t free_b = 0, total = 0;
+    if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return free_b >= needed + 9 * bytes;
+}
+
 int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const double* links,
                      double mass, unsigned flags) {
     if (!c || !out || !dims || !links) return MSC_ERR_ARG;
@@ -882,12 +897,20 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
     const bool unitary = dev[0] < 1e-9;
     d.recon = (!(flags & MSC_LINKS_FULL) && unitary && dev[1] < 1e-9) ? 1 : 0;
     const size_t l32 = d.recon ? (size_t)4 * V * (nc == 3 ? 3 : 1) * 16 : (size_t)4 * V * nc * nc * 8;
-    const size_t lfx = unitary ? (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16 : 0;
+    size_t lfx = unitary ? (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16 : 0;
+    if (lfx && !room_for_copy(lfx, nlink_bytes + l32)) lfx = 0;
     // one allocation for the three forms (each cudaMalloc and cudaFree costs
     // tens of microseconds of a small operator's set-up): FP64, limbs, FP32
-    const size_t at_fx = (nlink_bytes + 255) / 256 * 256, at_32 = at_fx + (lfx + 255) / 256 * 256;
+    const size_t at_fx = (nlink_bytes + 255) / 256 * 256;
+    size_t at_32 = at_fx + (lfx + 255) / 256 * 256;
     char* block = nullptr;
     e = cudaMalloc((void**)&block, at_32 + l32);
+    if (e == cudaErrorMemoryAllocation && lfx) {  // without the limbs, then
+        cudaGetLastError();
+        lfx = 0;
+        at_32 = at_fx;
+        e = cudaMalloc((void**)&block, at_32 + l32);
+    }
     if (e != cudaSuccess) return fail(e);
     d.links64 = (double2*)block;
     d.linksfx = lfx ? (int4*)(block + at_fx) : nullptr;
@@ -996,9 +1019,15 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
     if (e != cudaSuccess) return fail(cuda_status(e));
     if (bad & 1) return fail(MSC_ERR_ARG);
-    if (bd == 1 && !(bad & 4)) {
-        e = cudaMalloc((void**)&d.valsr, 8 * 32 * std::max<int64_t>(acc, 1));
-        if (e == cudaSuccess) e = bsr_pack_real(d, c->work);
+    const size_t lre = 8 * 32 * (size_t)std::max<int64_t>(acc, 1);
+    if (bd == 1 && !(bad & 4) && room_for_copy(lre, 0)) {
+        e = cudaMalloc((void**)&d.valsr, lre);
+        if (e == cudaErrorMemoryAllocation) {  // without the copy, then
+            cudaGetLastError();
+            d.valsr = nullptr;
+            e = cudaSuccess;
+        }
+        if (e == cudaSuccess && d.valsr) e = bsr_pack_real(d, c->work);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
         if (e != cudaSuccess) return fail(cuda_status(e));
     }
