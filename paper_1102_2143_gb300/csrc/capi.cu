@@ -893,11 +893,17 @@ int msc_op_staggered(msc_ctx* c, msc_op** out, int nc, const int dims[4], const 
     if (e == cudaSuccess) e = cudaMemcpyAsync(dev, ddev, sizeof dev, cudaMemcpyDeviceToHost, c->work);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
     if (e != cudaSuccess) return fail(e);
-    // limbs need entries of at most 1; rebuilding a row needs determinant 1 too
-    const bool unitary = dev[0] < 1e-9;
+    // Rebuilding a row needs determinant 1 too. Limbs need entries of at most 1,
+    // and links that couple every pair of colours: they hold an entry to 2^-57
+    // and sum a site's colours in one unit, so that an entry, or a colour that
+    // meets no other, far below 1 would keep fewer bits than in FP64 (unit links:
+    // a colour of 1e-20 beside one of 1 came out as 0). With the smallest entry
+    // of all at 2^-24 or more no colour's sum is that far below the unit alone; the
+    // smallest of the 4e7 entries of a random 32^4 field is about 1e-4.
+    const bool unitary = dev[0] < 1e-9, coupled = dev[2] <= 0x1p24;
     d.recon = (!(flags & MSC_LINKS_FULL) && unitary && dev[1] < 1e-9) ? 1 : 0;
     const size_t l32 = d.recon ? (size_t)4 * V * (nc == 3 ? 3 : 1) * 16 : (size_t)4 * V * nc * nc * 8;
-    size_t lfx = unitary ? (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16 : 0;
+    size_t lfx = unitary && coupled ? (size_t)4 * ((V + 31) / 32 * 32) * nc * nc * 16 : 0;
     if (lfx && !room_for_copy(lfx, nlink_bytes + l32)) lfx = 0;
     // one allocation for the three forms (each cudaMalloc and cudaFree costs
     // tens of microseconds of a small operator's set-up): FP64, limbs, FP32

@@ -53,7 +53,7 @@ struct OpDev {
     double mass;
     int recon;          // FP32 links keep nc-1 rows
     double2* links64;   // [4][nc*nc][V]
-    int4* linksfx;      // links in U(nc): fixed-point limbs (see fixed.cuh, fx_link); else null
+    int4* linksfx;      // links in U(nc) that couple the colours: fixed-point limbs (see fixed.cuh, fx_link); else null
     void* links32;      // full: float2 [4][nc*nc][V]; recon: float4 [4][k][V]
     // block-CSR in sliced-ELL form, 32 rows per slice
     int bd;
@@ -180,8 +180,8 @@ cudaError_t launch_norms(const Engine& e, const double2* v, int count, int64_t n
 // set-up kernels
 cudaError_t stag_pack_links(OpDev& op, const double2* links_aos, cudaStream_t st);
 // d_dev (zeroed by the caller): the links' deviations from U(nc) and from
-// determinant 1.
-constexpr int kLinkDevs = 2;
+// determinant 1, and the inverse of the smallest entry of all.
+constexpr int kLinkDevs = 3;
 cudaError_t stag_unitarity(const OpDev& op, const double2* links_aos, double* d_dev, cudaStream_t st);
 cudaError_t stag_pack_links32(OpDev& op, const double2* links_aos, cudaStream_t st);
 cudaError_t stag_pack_linksfx(OpDev& op, const double2* links_aos, cudaStream_t st);
