@@ -217,7 +217,9 @@ typedef struct {
                   and |r|^2 fused),
        update_ms  the fused multi-shift update kernel;
        prof_samples the number of samples (0: not measured, as on small
-                  staggered systems, whose iterations share one kernel);
+                  staggered systems, whose iterations share one kernel; a
+                  context created with MSC_PERSIST=0 in the environment runs
+                  and samples the per-pass kernels there too);
        prof_active  the mean, over the samples, of the number of non-base
                   shifts (summed over right-hand sides) still iterating at
                   the sampled iteration: the sampled update kernel moved

@@ -90,6 +90,7 @@ struct msc_ctx {
     int use_tile = 0;  // one-system FP32 stencil passes stage their links (when the lattice tiles)
     int test_no_copy = 0;  // tests only: the staged passes issue no copies, so their waits run out
     int test_absent = 0;   // tests only: grid barriers wait for an arrival that never comes
+    int use_persist = 1;  // small staggered stages iterate in one cooperative kernel
     int use_cond = 1; // build reliable updates as conditional graph nodes
     int* h_flags = nullptr;  // pinned copy of the conditional flags of a chunk
     int* h_act = nullptr;
@@ -564,7 +565,7 @@ static int run_stage(msc_ctx* c, const msc_op* op, int prec, int nsys, int chunk
     for (int j = 0; j < nsys; ++j) nslot_all = std::max(nslot_all, c->h_sys[j].slot0 + c->h_sys[j].S);
     const bool tiled = c->use_tile && nsys == 1 && prec == PREC_F32 && op->dev.kind == OP_STAGGERED && op->dev.recon &&
                        stag_tile_fits(op->dev.g, op->dev.nc);
-    if (!tiled && persist_applies(op->dev, prec, nsys, nslot_all))
+    if (c->use_persist && !tiled && persist_applies(op->dev, prec, nsys, nslot_all))
         return run_stage_persist(c, op, prec, nsys, nslot_all, reliable, npad, max_iter, rel_updates);
     GraphEntry* ge = nullptr;
     int st = MSC_OK;
@@ -729,6 +730,9 @@ int msc_create(msc_ctx** out, int device, void* stream) {
     // on the other blocks. For tests of the timeout paths only:
     // MSC_TEST_NO_COPY=1, the staged passes issue no copies; MSC_TEST_ABSENT=1,
     // the grid barriers wait for one arrival more than there are.
+    // MSC_PERSIST=0: small staggered stages run the per-pass kernels, whose times
+    // msc_info samples, instead of the cooperative one.
+    if (const char* ev = getenv("MSC_PERSIST")) c->use_persist = atoi(ev) != 0;
     if (const char* ev = getenv("MSC_STAG_TILE")) c->use_tile = atoi(ev) != 0;
     if (const char* ev = getenv("MSC_WAIT_NS")) {
         const long long w = atoll(ev);
