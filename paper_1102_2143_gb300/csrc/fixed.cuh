@@ -84,12 +84,18 @@ __device__ __forceinline__ int2 fx_unit(double u) {
     return q < 0 ? make_int2(-h, -l) : make_int2(h, l);
 }
 
+// The high word of a double (high word hi) times 2^(field - 1078 - half), field
+// an exponent in place. Unsigned: an ordinary result's exponent and field add
+// up to more than 2^31.
+__host__ __device__ __forceinline__ int fx_high(int hi, unsigned field, int half) {
+    return (int)((unsigned)hi + field - ((unsigned)(1078 + half) << 20));
+}
+
 // t units of the sum of products of unit factors and entries of exponent field
 // `field`, times 2^-half.
 __device__ __forceinline__ double fx_double(long long t, unsigned field, int half) {
     const double d = (double)t;
-    const int hi = __double2hiint(d) + (int)field - ((1078 + half) << 20);
-    return t == 0 ? 0.0 : __hiloint2double(hi, __double2loint(d));
+    return t == 0 ? 0.0 : __hiloint2double(fx_high(__double2hiint(d), field, half), __double2loint(d));
 }
 __device__ __forceinline__ double fx_value(const FxSum& s, unsigned field, int half) {
     return fx_double(s.h + ((s.m + (1 << 27)) >> 28), field, half);
