@@ -722,9 +722,11 @@ __global__ void k_packfx(const double2* __restrict__ in, int4* __restrict__ out,
 __device__ __forceinline__ double worse(double m, double d) { return d <= m ? m : d == d ? d : 1e300; }
 
 // dev[0]: max over links of |U U^dag - 1|_max, dev[1]: of |det U - 1|, dev[2]:
-// of 1 / (largest part of the link's smallest entry)
+// of 1 / (largest part of the link's smallest entry), to the bits of a high word
+// (integer minima: the FP64 pipe bounds this kernel)
 __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlinks, unsigned long long* dev) {
-    double m = 0.0, md = 0.0, mc = 0.0;
+    double m = 0.0, md = 0.0;
+    unsigned least = 0x7ff00000u;
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < nlinks;
          l += (int64_t)gridDim.x * blockDim.x) {
         const double2* u = in + l * nc * nc;
@@ -735,7 +737,11 @@ __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlin
                 if (a == b) s.x -= 1.0;
                 m = worse(worse(m, fabs(s.x)), fabs(s.y));
             }
-        for (int q = 0; q < nc * nc; ++q) mc = worse(mc, 1.0 / worse(fabs(u[q].x), fabs(u[q].y)));
+        for (int q = 0; q < nc * nc; ++q) {
+            unsigned e = 0;
+            fx_bound(e, u[q]);
+            least = min(least, e);
+        }
         double2 det;
         if (nc == 2) {
             det = csub(cmul(u[0], u[3]), cmul(u[1], u[2]));
@@ -752,7 +758,7 @@ __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlin
     // 27,000-site SU(2) operator 0.2 ms longer)
     unsigned long long b[kLinkDevs] = {(unsigned long long)__double_as_longlong(m),
                                        (unsigned long long)__double_as_longlong(md),
-                                       (unsigned long long)__double_as_longlong(mc)};
+                                       (unsigned long long)__double_as_longlong(1.0 / __hiloint2double((int)least, 0))};
     for (int k = 0; k < kLinkDevs; ++k) {
         for (int o = 16; o > 0; o >>= 1) b[k] = max(b[k], __shfl_xor_sync(0xffffffffu, b[k], o));
         if ((threadIdx.x & 31) == 0) atomicMax(dev + k, b[k]);
