@@ -58,6 +58,8 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
     int found = 0;
     for (int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; row < nrow_pad;
          row += (int64_t)gridDim.x * blockDim.x) {
+        // limbs that will not be used: the packing is repeated without them
+        if (vfx && (*(volatile int*)bad & 2)) break;
         const int64_t slice = row >> 5;
         const int lane = (int)(row & 31);
         const int len = slice_len[slice];
@@ -75,14 +77,16 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
                 if (c < 0 || (int64_t)c >= nbr) { found |= 1; c = 0; }
             }
             pcol[slot * 32 + lane] = c;
+            double2 blk[e2];
+#pragma unroll
+            for (int q = 0; q < e2; ++q) blk[q] = k < rl ? vals[(b0 + k) * e2 + q] : double2{0.0, 0.0};
             int ex = 0;
             if (vfx) {
                 unsigned e = 0;
                 bool zero = true;
 #pragma unroll
                 for (int q = 0; q < e2; ++q) {
-                    if (k >= rl) continue;
-                    const double2 v = vals[(b0 + k) * e2 + q];
+                    const double2 v = blk[q];
                     fx_bound(part[q], v);
                     fx_bound(e, v);
                     zero = zero && v.x == 0.0 && v.y == 0.0;
@@ -93,8 +97,7 @@ __global__ void k_bsr_pack(const int64_t* __restrict__ row_ptr, const int32_t* _
             }
 #pragma unroll
             for (int q = 0; q < e2; ++q) {
-                double2 v = {0.0, 0.0};
-                if (k < rl) v = vals[(b0 + k) * e2 + q];
+                const double2 v = blk[q];
                 if (bd == 1 && !(v.y == 0.0)) found |= 4;
                 if (v64) v64[(slot * e2 + q) * 32 + lane] = v;
                 v32[(slot * e2 + q) * 32 + lane] = make_float2((float)v.x, (float)v.y);

@@ -1041,15 +1041,17 @@ int msc_op_bsr(msc_ctx* c, msc_op** out, int64_t nbr, int bd, const int64_t* row
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
         if (e != cudaSuccess) return fail(cuda_status(e));
     }
-    if (bad & 2) {  // some block does not fit the limbs: the whole matrix in FP64
+    if (bad & 2) {  // some block row does not fit the limbs: the whole matrix in FP64
         cudaFree(d.valsfx);
         cudaFree(d.blkfx);
         d.valsfx = nullptr;
         d.blkfx = nullptr;
         e = cudaMalloc((void**)&d.vals64, 16 * e2 * 32 * std::max<int64_t>(acc, 1));
         if (e == cudaSuccess) e = bsr_pack(d, (const int64_t*)trp, dcol, dval, dbad, c->work);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, dbad, sizeof(int), cudaMemcpyDeviceToHost, c->work);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->work);
         if (e != cudaSuccess) return fail(cuda_status(e));
+        if (bad & 1) return fail(MSC_ERR_ARG);  // in rows that the first packing left out
     }
     if (flags & MSC_CHECK_HERMITIAN) {
         // the columns are known to be in range now (the packing checked them)

@@ -198,7 +198,8 @@ cudaError_t bsr_pack_real(OpDev& op, cudaStream_t st);
 // bit 0 of *d_bad on a column out of range, bit 1 on a block row that limbs
 // cannot hold (entries that are not finite, near the ends of the exponent
 // range, or far smaller than others of their block row) and bit 2 on an entry
-// that is not real.
+// that is not real. Once bit 1 is set, rows may be left out (all of them are
+// packed, and their columns checked, when valsfx is null).
 cudaError_t bsr_pack(OpDev& op, const int64_t* d_row_ptr, const int32_t* d_col,
                      const double2* d_vals, int* d_bad, cudaStream_t st);
 

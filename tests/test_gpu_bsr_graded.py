@@ -102,3 +102,19 @@ def test_reported_residual_is_the_given_matrix(ctx, big):
         assert abs(rho - rep[s]) <= 1e-12, (sg, rho, rep[s])
         if info.status == 0:
             assert rho <= 1.01e-10
+
+
+def test_bad_column_behind_a_graded_row_is_refused(ctx):
+    """A column out of range in the last row, with a first row that sends the
+    matrix to FP64 before the last is looked at."""
+    bd, nbr = 2, 200000
+    rp = np.arange(nbr + 1, dtype=np.int64)
+    ci = np.arange(nbr, dtype=np.int32)
+    va = np.tile(np.array([[2.0, 1.0], [1.0, 2.0]], complex), (nbr, 1, 1))
+    va[0] = np.diag([1e12, 1.0])
+    op = msc.msc_op_bsr(ctx, nbr, bd, rp, ci, va)
+    msc.msc_op_destroy(op)
+    ci[-1] = nbr
+    with pytest.raises(msc.MscError) as e:
+        msc.msc_op_bsr(ctx, nbr, bd, rp, ci, va)
+    assert e.value.code == msc.MSC_ERR_ARG
