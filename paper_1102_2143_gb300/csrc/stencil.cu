@@ -755,13 +755,14 @@ __global__ void k_unitarity(const double2* __restrict__ in, int nc, int64_t nlin
     }
     // non-negative doubles order like their bit patterns; one atomic per warp
     // (one per link on one address made it 200 us at 16^4, and the set-up of a
-    // 27,000-site SU(2) operator 0.2 ms longer)
+    // 27,000-site SU(2) operator 0.2 ms longer), left out where a larger value is
+    // already there
     unsigned long long b[kLinkDevs] = {(unsigned long long)__double_as_longlong(m),
                                        (unsigned long long)__double_as_longlong(md),
                                        (unsigned long long)__double_as_longlong(1.0 / __hiloint2double((int)least, 0))};
     for (int k = 0; k < kLinkDevs; ++k) {
         for (int o = 16; o > 0; o >>= 1) b[k] = max(b[k], __shfl_xor_sync(0xffffffffu, b[k], o));
-        if ((threadIdx.x & 31) == 0) atomicMax(dev + k, b[k]);
+        if ((threadIdx.x & 31) == 0 && b[k] > *(volatile unsigned long long*)(dev + k)) atomicMax(dev + k, b[k]);
     }
 }
 
