@@ -182,8 +182,8 @@ __device__ __forceinline__ void bsr_row_fx(const OpDev& A, const double2* __rest
             const double scale = __hiloint2double((top - 1077) << 20, 0);
 #pragma unroll
             for (int a = 0; a < BD; ++a) {
-                y[a].x = fma((double)(re[a].h + (re[a].m >> 28)), scale, y[a].x);
-                y[a].y = fma((double)(im[a].h + (im[a].m >> 28)), scale, y[a].y);
+                y[a].x = fma((double)fx_units(re[a]), scale, y[a].x);
+                y[a].y = fma((double)fx_units(im[a]), scale, y[a].y);
             }
         } else if (!finite || top != 0) {
             RowVec<BD> r;

@@ -97,8 +97,10 @@ __device__ __forceinline__ double fx_double(long long t, unsigned field, int hal
     const double d = (double)t;
     return t == 0 ? 0.0 : __hiloint2double(fx_high(__double2hiint(d), field, half), __double2loint(d));
 }
+// The sum in units, rounded.
+__device__ __forceinline__ long long fx_units(const FxSum& s) { return s.h + ((s.m + (1 << 27)) >> 28); }
 __device__ __forceinline__ double fx_value(const FxSum& s, unsigned field, int half) {
-    return fx_double(s.h + ((s.m + (1 << 27)) >> 28), field, half);
+    return fx_double(fx_units(s), field, half);
 }
 
 }  // namespace msc

@@ -442,7 +442,7 @@ __device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeo
     long long sr = 0, si = 0;
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
-        long long r = re[a].h + ((re[a].m + (1 << 27)) >> 28), i = im[a].h + ((im[a].m + (1 << 27)) >> 28);
+        long long r = fx_units(re[a]), i = fx_units(im[a]);
         r += __shfl_xor_sync(0xffffffffu, r, 1);
         i += __shfl_xor_sync(0xffffffffu, i, 1);
         r += __shfl_xor_sync(0xffffffffu, r, 2);
