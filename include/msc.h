@@ -57,7 +57,12 @@ extern "C" {
 #define MSC_ERR_BREAKDOWN     9  /* msc_solve_nonherm: a BiCGStab denominator vanished */
 
 /* precision of the iteration */
-#define MSC_FP64  0  /* every vector, link, block and scalar in FP64 */
+#define MSC_FP64  0  /* every vector and scalar in FP64. Operator sums: in FP64,
+                        or, where the links or blocks allow it (see
+                        msc_op_staggered, msc_op_bsr), in fixed point with 56
+                        bits below the largest entry that meets in a sum;
+                        2-norm errors are then at or below those of FP64
+                        sums, terms far below the largest keep fewer bits */
 #define MSC_MIXED 1  /* FP32 operator and vector updates; FP64 zeta/alpha/beta
                         recurrences, FP64 dot-product accumulation, FP64
                         reliable updates of the base residual and FP64
@@ -92,7 +97,11 @@ int msc_set_stream(msc_ctx* ctx, void* cuda_stream);
  * U[mu][site][a][b]. A vector is [V][nc] complex. Unless MSC_LINKS_FULL is
  * given, FP32 links keep nc-1 rows and rebuild the last one from unitarity
  * when every link is in SU(nc) to 1e-9 (checked on the device); otherwise
- * all entries are kept. */
+ * all entries are kept. The FP64 passes sum in fixed point when every link is
+ * in U(nc) to 1e-9, no entry of any link is below 2^-24 (links that are diagonal
+ * or nearly so keep the FP64 sums, componentwise) and the device has room for
+ * that second copy of the links beside the solves (a copy above 64 MB is made
+ * only where eight times its size stays free). */
 int msc_op_staggered(msc_ctx* ctx, msc_op** op, int nc, const int dims[4],
                      const double* links, double mass, unsigned flags);
 
@@ -110,7 +119,12 @@ int msc_op_staggered(msc_ctx* ctx, msc_op** op, int nc, const int dims[4],
  * against a zero partner); its cost is, per stored block, the length of
  * its row and of its column's row. Without the flag Hermiticity is not
  * checked; positivity is never checked here (the solve reports
- * MSC_ERR_NOT_HPD when it meets p^dagger A p <= 0). n = nbr * bd. A block
+ * MSC_ERR_NOT_HPD when it meets p^dagger A p <= 0). bd = 2 and 3: the FP64
+ * passes sum in fixed point when in every block row each component's row and
+ * column has an entry within 2^-4 of the row's largest and each pair of
+ * components one within 2^-24; otherwise, and where an entry is not finite or
+ * near the ends of the exponent range, the whole matrix keeps its FP64 entries
+ * and sums. n = nbr * bd. A block
  * row may hold at most 2^26 / (bd * bd) blocks (about 7.4 million 3 x 3
  * blocks); longer rows, like any other malformed input, give MSC_ERR_ARG. */
 int msc_op_bsr(msc_ctx* ctx, msc_op** op, int64_t nbr, int bd, const int64_t* row_ptr,

@@ -63,7 +63,8 @@ __device__ __forceinline__ void bsr_row_real(const OpDev& A, const double2* __re
 }
 
 // ---------------------------------------------------------------------------
-// FP64 rows by fixed-point sums (fixed.cuh), bd = 2 and 3. A block is stored as
+// FP64 rows by fixed-point sums (fixed.cuh), bd = 2 and 3, for matrices whose
+// block rows hold entries of like sizes (bsr_even_row, bsr.cu). A block is stored as
 // the 28-bit limbs of its entries in units of 2^-56 of the power of two above
 // its largest part (valsfx, [slot][component][lane]) and that exponent (blkfx,
 // [slot][lane], biased; 0: a zero block). G blocks of a row share one

@@ -7,18 +7,26 @@
 // sum_k u_k v_k is formed in fixed point instead:
 //
 //   - every factor is a signed 56-bit integer in units of 2^-56 of a power of
-//     two that bounds its group (links: 1; the vector entries that one output
-//     needs: the largest of their exponents), kept as two 28-bit limbs of the
-//     value's sign, x = h 2^28 + l;
+//     two that bounds its group (links: 1; block-CSR: the block's largest part;
+//     the vector entries that one output needs: the largest of them), kept as
+//     two 28-bit limbs of the value's sign, x = h 2^28 + l;
 //   - u v = uh vh 2^56 + (uh vl + ul vh) 2^28 + ul vl, with the last term
-//     dropped: three multiply-adds into two 64-bit sums, exact;
+//     dropped: three multiply-adds into two 64-bit sums that lose nothing more;
 //   - the sums go back to FP64 once per output, rounded once.
 //
-// Error of an output against the exact sum, with v_max the bound of its
-// vector entries: the quantisation of u and v (2^-56 each, at most) and the
-// dropped term (2^-56 per product) are about 2^-56 |u| v_max sqrt(terms) in
-// all; 48 chained DFMAs round to about 2^-54 of their partial sums each.
-// Measured: see tests/test_gpu_fixed_fp64.py.
+// Error of an output against the exact sum. With B the power of two above the
+// largest part of the vector entries that the site gathers (twice that where the
+// stencil spares a bit), each product adds at most 2^-57 B (the link part,
+// rounded), 2^-56 B |u| (the entry, truncated) and 2^-56 B (the dropped term);
+// independent, about 2^-56 B sqrt(terms) together. 48 chained DFMAs round to
+// about 2^-54 of their partial sums each. Block-CSR: the same per group of
+// blocks, B the largest product of a block's and its entries' powers of two.
+// These bounds are relative to the largest entry or product that meets in a sum,
+// not to each term, as FP64 roundings are: a term far below the largest keeps
+// fewer bits. So the form is taken only where the matrix itself leaves no output
+// to such terms alone: links that couple every pair of colours (within 2^-24,
+// msc_op_staggered), block rows of like sizes (bsr_even_row). The 2-norm errors
+// are at or below FP64's (tests/test_gpu_fixed_fp64.py).
 //
 // Range of the 64-bit sums: |uh vh| <= 2^56 and |uh vl| + |ul vh| <= 2^57 per
 // product, so up to 48 products (48 2^57 < 2^62.6) cannot overflow.

@@ -14,8 +14,10 @@
 //
 // A launch ends when every system has stopped, when one is due a reliable
 // update, or after a number of iterations; block 0 then stores the scalars.
-// The sums are those of k_stag for one system (one site per thread, a partial
-// per 256 sites), so a solve gives the same bits either way.
+// The sums are those of the per-pass kernels up to their order and to where
+// they are rounded (here one site per thread and a partial per 256 sites, or 64
+// with four lanes a site), so that a solve by either agrees to rounding, not in
+// its bits.
 //
 // Measured, one system, mixed, per iteration: 4^4 with 8 shifts 37 -> 12 us,
 // 16^4 with one shift 29 -> 18 us (of which three barriers 3.8, the scalar

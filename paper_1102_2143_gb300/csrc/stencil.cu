@@ -70,8 +70,8 @@ k_stag(Engine e, const PassDesc* descs, int npass, const int* act, StagGeom g, c
 }
 
 // (descs null: the single pass `one`, a kernel parameter.)
-// The FP64 pass over unitary links by fixed-point sums (dslash_site_fx; links
-// that are not unitary may have any range and keep k_stag<double>). Four
+// The FP64 pass over links in U(nc) that couple the colours by fixed-point sums
+// (dslash_site_fx; other links may have any range and keep k_stag<double>). Four
 // 128-thread blocks per SM at 128 registers: three at 168 take 2% longer and
 // five at 96 spill. 32^4, one system: 204 us per pass against 570 us on the
 // FP64 pipe (3.9 TB/s against 1.4); about 1,350 instructions per site on the

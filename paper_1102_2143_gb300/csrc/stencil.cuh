@@ -217,7 +217,7 @@ __host__ __device__ __forceinline__ size_t fx_link(int mu, int x, int V) {
 // loads do not take the read-only path.
 template <int NC, bool FRESH>
 __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* links64, const double2* src, int x, const StagGeom& g, double2 (&y)[NC]) {
-    if (!lfx) {  // links that are not unitary (batches mix operators)
+    if (!lfx) {  // links without limbs (batches mix operators)
         const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g, false);
 #pragma unroll
         for (int a = 0; a < NC; ++a) y[a] = r.y[a];
