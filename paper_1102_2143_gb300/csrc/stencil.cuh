@@ -160,39 +160,37 @@ __device__ __forceinline__ void dslash_site(const void* links, const T2<T>* __re
 }
 
 // y = D src at site x in FP64 on the FP64 pipe, for the sites whose entries
-// leave the range of the fixed-point sums (rare: out of line). finite: the
-// links are, so a site whose entries are all zero has y = 0 without the sums: a
-// source on one site or one parity stays on alternating parities under D, and
-// half the lanes of every warp of an FP64 pass then come here.
+// leave the range of the fixed-point sums (rare: out of line).
 template <int NC> struct SiteVec {
     double2 y[NC];
 };
 template <int NC>
-__device__ __noinline__ SiteVec<NC> dslash_site_f64(const void* links64, const double2* src, int x, const StagGeom& g,
-                                                    bool finite) {
+__device__ __noinline__ SiteVec<NC> dslash_site_f64(const void* links64, const double2* src, int x, const StagGeom& g) {
     SiteVec<NC> r;
-    unsigned long long bits = finite ? 0 : 1;
-    if (finite) {
-        const SiteNbrs nb = neighbours(x, g);
+    dslash_site_fresh<double, NC, 0>(links64, src, x, g, r.y);
+    return r;
+}
+
+// Whether every entry that site x gathers is zero: y = 0 then without the sums,
+// as the links are finite. A source on one site or one parity stays on
+// alternating parities under D, and half the lanes of every warp of an FP64 pass
+// then ask.
+template <int NC>
+__device__ __noinline__ bool site_among_zeros(const double2* src, int x, const StagGeom& g) {
+    const SiteNbrs nb = neighbours(x, g);
+    unsigned long long bits = 0;
 #pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            const double2* vf = src + (size_t)vsite(nb.fwd[mu], g) * NC;
-            const double2* vb = src + (size_t)vsite(nb.bwd[mu], g) * NC;
+    for (int mu = 0; mu < 4; ++mu) {
+        const double2* vf = src + (size_t)vsite(nb.fwd[mu], g) * NC;
+        const double2* vb = src + (size_t)vsite(nb.bwd[mu], g) * NC;
 #pragma unroll
-            for (int b = 0; b < NC; ++b) {
-                const double2 f = vf[b], w = vb[b];
-                bits |= (unsigned long long)(__double_as_longlong(f.x) | __double_as_longlong(f.y) |
-                                             __double_as_longlong(w.x) | __double_as_longlong(w.y)) << 1;
-            }
+        for (int b = 0; b < NC; ++b) {
+            const double2 f = vf[b], w = vb[b];
+            bits |= (unsigned long long)(__double_as_longlong(f.x) | __double_as_longlong(f.y) |
+                                         __double_as_longlong(w.x) | __double_as_longlong(w.y)) << 1;
         }
     }
-    if (bits) {
-        dslash_site_fresh<double, NC, 0>(links64, src, x, g, r.y);
-    } else {
-#pragma unroll
-        for (int a = 0; a < NC; ++a) r.y[a] = {0.0, 0.0};
-    }
-    return r;
+    return bits == 0;
 }
 
 // Index of entry 0 of link (mu, x) in the limb array: sites in groups of 32,
@@ -218,7 +216,7 @@ __host__ __device__ __forceinline__ size_t fx_link(int mu, int x, int V) {
 template <int NC, bool FRESH>
 __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* links64, const double2* src, int x, const StagGeom& g, double2 (&y)[NC]) {
     if (!lfx) {  // links without limbs (batches mix operators)
-        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g, false);
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
 #pragma unroll
         for (int a = 0; a < NC; ++a) y[a] = r.y[a];
         return;
@@ -281,7 +279,12 @@ __device__ __forceinline__ void dslash_site_fx(const void* lfx, const void* link
         }
     }
     if (!fx_in_range(field)) {
-        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g, true);
+        if (site_among_zeros<NC>(src, x, g)) {
+#pragma unroll
+            for (int a = 0; a < NC; ++a) y[a] = {0.0, 0.0};
+            return;
+        }
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
 #pragma unroll
         for (int a = 0; a < NC; ++a) y[a] = r.y[a];
         return;
@@ -454,7 +457,7 @@ __device__ __forceinline__ double stag_site_fx4(const PassDesc& d, const StagGeo
     if (e == 0) {
         y = {0.0, 0.0};
     } else if (!fx_in_range(field)) {
-        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g, false);
+        const SiteVec<NC> r = dslash_site_f64<NC>(links64, src, x, g);
 #pragma unroll
         for (int a = 0; a < NC; ++a)
             if (a == mu) y = r.y[a];

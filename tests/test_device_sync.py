@@ -32,7 +32,8 @@ def test_vectors_that_other_blocks_write_are_not_read_as_constant():
     the same kernel wrote: the functions on that path hold them in plain
     pointers, and the read-only path is for links or for FRESH = false."""
     text = dict(sources())["stencil.cuh"]
-    for fn in ("dslash_site_fresh", "dslash_site_f64", "dslash_site_fx", "stag_colour_of", "stag_site", "stag_site_fx4"):
+    for fn in ("dslash_site_fresh", "dslash_site_f64", "site_among_zeros", "dslash_site_fx", "stag_colour_of", "stag_site",
+               "stag_site_fx4"):
         at = re.search(r"__device__ \w+ (?:SiteAcc<T, KIND>|SiteVec<NC>|\w+) " + fn + r"\(", text).start()
         end = text.find("\ntemplate", at)
         body = text[at:end if end > 0 else None]
